@@ -61,3 +61,30 @@ def test_adam_matches_oracle():
         N.ddps_mlp_adam(p, g, m, v, p.numel(), 1e-2, 0.9, 0.999, 1e-8, step)
         M.adam_step(params, grads, state, lr=1e-2)
     assert np.max(np.abs(p.cpu().numpy() - _flat(params))) <= 1e-5
+
+
+@pytest.mark.parametrize("d_in,hidden,layers,d_out,B", [
+    (1, 256, 3, 129, 1),      # one vector: a warp per four rows, a ragged last group
+    (2, 33, 2, 130, 4),       # rows that are not 16-byte aligned
+    (2, 256, 3, 2500, 5),     # the smallest batch of the tiled products
+    (3, 48, 1, 31, 64),       # one hidden layer, every product small
+    (2, 256, 3, 5003, 100),   # wide output: K splits with a remainder, ragged tiles
+    (2, 300, 2, 1024, 130),   # more than one K stage of the small product
+])
+def test_shapes_match_oracle(d_in, hidden, layers, d_out, B):
+    """Forward and gradients at the edges of the kernels' tiles: sums of at most
+    5,003 FP32 products, whose rounding stays below 1e-5 of the result's norm."""
+    params, X, T, _ = _setup(3, d_in, hidden, layers, d_out, B)
+    p = _dev(_flat(params))
+    ws = torch.empty(N.ddps_mlp_workspace_bytes(d_in, hidden, layers, d_out, B), dtype=torch.uint8,
+                     device="cuda")
+    Y = torch.empty(B, d_out, dtype=torch.float32, device="cuda")
+    N.ddps_mlp_forward(p, d_in, hidden, layers, d_out, _dev(X), B, Y, ws)
+    Yo, _ = M.forward(params, X)
+    assert np.linalg.norm(Y.cpu().numpy() - Yo) <= 1e-5 * np.linalg.norm(Yo)
+    g = torch.full_like(p, float("nan"))
+    loss = torch.zeros(1, dtype=torch.float32, device="cuda")
+    N.ddps_mlp_backward(p, d_in, hidden, layers, d_out, _dev(X), _dev(T), B, g, loss, ws)
+    go = _flat(M.backward(params, X, T))
+    assert np.linalg.norm(g.cpu().numpy() - go) <= 1e-5 * np.linalg.norm(go)
+    assert abs(loss.item() - M.loss(params, X, T)) <= 1e-5 * M.loss(params, X, T)
