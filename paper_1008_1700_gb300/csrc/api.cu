@@ -22,6 +22,7 @@
 
 #include "ddps.h"
 #include "ddps_internal.h"
+#include "inner_cluster.h"
 #include "krylov.h"
 #include "launch.h"
 #include "reduced_direct.h"
@@ -245,6 +246,8 @@ struct ddps_handle {
   // most kPersistM rows): orders, waits and flags (2 nfronts done flags, 2 counters)
   int32_t persist_L = -1, persist_n = 0, persist_max_m = 0;
   int32_t *p_fwd = nullptr, *p_bwd = nullptr, *p_wait = nullptr, *p_flags = nullptr;
+  // the inner BiCGStab of small systems in one launch (inner.ok false: a system is too large)
+  InnerPlan inner;
   // direct solve of the reduced system (reduced_solver DIRECT)
   DirectPlan direct;
   bool use_direct = false;
@@ -1008,7 +1011,7 @@ RedSpec nored() { return RedSpec{nullptr, nullptr, 0, 0, nullptr}; }
 // ---------------------------------------------------------------------------
 template <typename TG, typename TI>
 double inner_solve(ddps_handle* h, const double* ghat64, double* zhat64, const double* z0,
-                   cudaStream_t s) {
+                   cudaStream_t s, bool masked) {
   const int64_t m = (int64_t)h->A.c.size();
   const SegView& S = h->Sm;
   const int ns = h->nseg;
@@ -1019,6 +1022,23 @@ double inner_solve(ddps_handle* h, const double* ghat64, double* zhat64, const d
     explicit HostScalars(ddps_handle* hh) : h(hh), saved(hh->hsc) { h->hsc = h->hsc_in; }
     ~HostScalars() { h->hsc = saved; }
   } host_scalars(h);
+  if (h->inner.ok) {  // every system fits the shared memory of a cluster
+    {
+      Prof pr(h, DDPS_PROF_GHAT_MATVEC, s);
+      h->launches += launch_inner_cluster<TG, TI>(h->inner, (const TG*)h->ghat, ghat64, z0, zhat64,
+                                                  sc, masked ? h->sc_out : nullptr, h->opt.tol_in,
+                                                  h->opt.maxit_in, s);
+    }
+    download_sc(h, sc, s);
+    double mx = 0.0;
+    for (int q = 0; q < ns; ++q) {
+      mx = std::max(mx, h->hsc[q].iters);
+      if (h->hsc[q].flag) h->stat_guess_used = true;
+    }
+    if (h->prof_mask & (1 << DDPS_PROF_GHAT_MATVEC))  // the products inside the launch
+      h->prof_cnt[DDPS_PROF_GHAT_MATVEC] += std::max<int64_t>((int64_t)std::ceil(2.0 * mx) - 1, 0);
+    return mx;
+  }
   TI *g = (TI*)h->i_g, *z = (TI*)h->i_z, *r = (TI*)h->i_r, *rh = (TI*)h->i_rh, *p = (TI*)h->i_p,
      *v = (TI*)h->i_v, *sv = (TI*)h->i_s, *t = (TI*)h->i_t;
   convert<TI, double>(m, ghat64, g, s);
@@ -1034,7 +1054,7 @@ double inner_solve(ddps_handle* h, const double* ghat64, double* zhat64, const d
   std::vector<double> iters(ns, 0.0);
   for (int q = 0; q < ns; ++q) {
     KScal& k = h->hsc[q];
-    k.active = k.ref > 0.0;
+    k.active = k.ref > 0.0 && !(masked && !h->hsc_out[q].active);
     k.flag = 0;
     k.half_done = 0;
     k.rho_old = k.alpha = k.omega = 1.0;
@@ -1172,19 +1192,21 @@ double inner_solve(ddps_handle* h, const double* ghat64, double* zhat64, const d
   return mx;
 }
 
+// masked: called by the outer iteration, whose finished systems (sc_out) are skipped: their
+// preconditioned vectors are not read.
 double inner_dispatch(ddps_handle* h, const double* ghat64, double* zhat64, const double* z0,
-                      cudaStream_t s) {
+                      cudaStream_t s, bool masked) {
   NvtxRange nv("reduced_solve");
   const int gp = h->opt.ghat_prec, ip = h->opt.inner_prec;
-  if (gp == DDPS_FP64) return inner_solve<double, double>(h, ghat64, zhat64, z0, s);
+  if (gp == DDPS_FP64) return inner_solve<double, double>(h, ghat64, zhat64, z0, s, masked);
   if (gp == DDPS_FP32)
-    return ip == DDPS_FP64 ? inner_solve<float, double>(h, ghat64, zhat64, z0, s)
-                           : inner_solve<float, float>(h, ghat64, zhat64, z0, s);
+    return ip == DDPS_FP64 ? inner_solve<float, double>(h, ghat64, zhat64, z0, s, masked)
+                           : inner_solve<float, float>(h, ghat64, zhat64, z0, s, masked);
   if (gp == DDPS_FP16)
-    return ip == DDPS_FP64 ? inner_solve<__half, double>(h, ghat64, zhat64, z0, s)
-                           : inner_solve<__half, float>(h, ghat64, zhat64, z0, s);
-  return ip == DDPS_FP64 ? inner_solve<__nv_bfloat16, double>(h, ghat64, zhat64, z0, s)
-                         : inner_solve<__nv_bfloat16, float>(h, ghat64, zhat64, z0, s);
+    return ip == DDPS_FP64 ? inner_solve<__half, double>(h, ghat64, zhat64, z0, s, masked)
+                           : inner_solve<__half, float>(h, ghat64, zhat64, z0, s, masked);
+  return ip == DDPS_FP64 ? inner_solve<__nv_bfloat16, double>(h, ghat64, zhat64, z0, s, masked)
+                         : inner_solve<__nv_bfloat16, float>(h, ghat64, zhat64, z0, s, masked);
 }
 
 // Fig. 3 with the direct reduced solve: a fixed launch sequence for given
@@ -1192,7 +1214,8 @@ double inner_dispatch(ddps_handle* h, const double* ghat64, double* zhat64, cons
 void precond_direct_launches(ddps_handle* h, const double* y, double* z, cudaStream_t s);
 
 // Fig. 3: z = P^-1 y.
-void precond_apply(ddps_handle* h, const double* y, double* z, cudaStream_t s, bool first) {
+void precond_apply(ddps_handle* h, const double* y, double* z, cudaStream_t s, bool first,
+                   bool masked) {
   const int64_t m = (int64_t)h->A.c.size();
   if (h->use_direct && m > 0) {
     if (graphs_on(h)) {
@@ -1227,7 +1250,7 @@ void precond_apply(ddps_handle* h, const double* y, double* z, cudaStream_t s, b
   launch_gather(h->pc_g, h->c, m, h->pc_ghat, s);                        // 6.2
   h->launches++;
   const double* z0 = (first && h->has_guess) ? h->guess : nullptr;
-  const double its = inner_dispatch(h, h->pc_ghat, h->pc_zhat, z0, s);  // 6.3
+  const double its = inner_dispatch(h, h->pc_ghat, h->pc_zhat, z0, s, masked);  // 6.3
   h->stat_inner += (int64_t)std::ceil(its);
   if (first) {
     h->stat_first_inner = its;
@@ -1325,7 +1348,7 @@ ddps_status solve_impl(ddps_handle* h, const double* f, double* x, const double*
     sc_beta(ns, sc, it == 1, s);
     update_p<double>(S, sc, h->o_r, h->o_p, h->o_v, s);
     h->launches += 4;
-    precond_apply(h, h->o_p, h->o_phat, s, first);
+    precond_apply(h, h->o_p, h->o_phat, s, first, true);
     first = false;
     spmv(h->o_phat, h->o_v);
     seg_reduce<double>(S, 1, red(h->o_rhat, h->o_v, 0, &sc[0].sigma), nored(), nored(), h->partial, s);
@@ -1366,7 +1389,7 @@ ddps_status solve_impl(ddps_handle* h, const double* f, double* x, const double*
       upload_sc(h, sc, s);
     }
     if (!any_active()) break;
-    precond_apply(h, h->o_s, h->o_shat, s, false);
+    precond_apply(h, h->o_s, h->o_shat, s, false, true);
     spmv(h->o_shat, h->o_t);
     seg_reduce<double>(S, 2, red(h->o_t, h->o_s, 0, &sc[0].ts), red(h->o_t, h->o_t, 0, &sc[0].tt),
                        nored(), h->partial, s);
@@ -2014,11 +2037,33 @@ void build_device(ddps_handle* h, const int32_t* rowptr, const int32_t* colind) 
       h->p_flags = dalloc<int32_t>(h, 2 * nf + 2);
     }
   }
+  std::vector<int32_t> gcols_panel(A.gcols.size());
+  for (int32_t b = 0; b < A.p; ++b)
+    for (int64_t pc = A.gcol_ptr[b]; pc < A.gcol_ptr[b + 1]; ++pc)
+      gcols_panel[pc] = A.gcols[A.gcol_ptr[b] + h->gperm[pc]];
+  if (h->opt.reduced_solver == DDPS_REDUCED_ITERATIVE && m > 0 && !implicit) {
+    InnerInput in;
+    in.nsys = A.nsys;
+    in.sys_c_ptr = A.sys_c_ptr.data();
+    in.sys_block_ptr = A.sys_block_ptr.data();
+    in.gq0 = A.gq0.data();
+    in.gq1 = A.gq1.data();
+    in.gcol_ptr = A.gcol_ptr.data();
+    in.ghat_off = A.ghat_off.data();
+    in.gld = A.gld.data();
+    in.gcols_panel = gcols_panel.data();
+    in.nsm = device_sm_count();
+    in.size_g = (int32_t)prec_size(h->opt.ghat_prec);
+    in.size_acc = h->opt.ghat_prec == DDPS_FP64 ? 8 : 4;
+    in.size_i = (int32_t)prec_size(h->opt.inner_prec);
+    plan_inner_cluster(in, h->inner);
+    if (h->inner.ok) {
+      h->inner.ctas = dupload(h, h->inner.h_ctas);
+      h->inner.groups = dupload(h, h->inner.h_groups);
+      h->inner.cols = dupload(h, h->inner.h_cols);
+    }
+  }
   if (h->opt.reduced_solver == DDPS_REDUCED_DIRECT && m > 0) {
-    std::vector<int32_t> gcols_panel(A.gcols.size());
-    for (int32_t b = 0; b < A.p; ++b)
-      for (int64_t pc = A.gcol_ptr[b]; pc < A.gcol_ptr[b + 1]; ++pc)
-        gcols_panel[pc] = A.gcols[A.gcol_ptr[b] + h->gperm[pc]];
     DirectInput in;
     in.p = A.p;
     in.m = m;
@@ -2404,7 +2449,7 @@ ddps_status ddps_reduced_solve(ddps_handle* h, const double* ghat, double* zhat,
       h->launches += direct_solve(h->direct, ghat, zhat, s);
     } else {
       h->stat_inner = 0;
-      inner_dispatch(h, ghat, zhat, nullptr, s);
+      inner_dispatch(h, ghat, zhat, nullptr, s, false);
     }
     check_launch();
   } catch (const Fail& e) {
@@ -2418,7 +2463,7 @@ ddps_status ddps_precond_apply(ddps_handle* h, const double* y, double* z, void*
   if (!h->factored) return DDPS_ERR_STATE;
   try {
     h->stat_inner = 0;
-    precond_apply(h, y, z, as_stream(stream), false);
+    precond_apply(h, y, z, as_stream(stream), false, false);
     check_launch();
   } catch (const Fail& e) {
     return fail(h, e);

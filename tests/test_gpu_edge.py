@@ -131,3 +131,34 @@ def test_direct_chain_with_a_one_sided_coupling():
     zo, _ = o.reduced_solve(g, mode="direct")
     assert relerr(host(S.reduced_solve(dev(g))), zo) <= 1e-4
     S.close()
+
+
+@pytest.mark.parametrize("name,N_,p,form", [
+    ("one_cta", 12, 3, "half"),          # a single CTA holds the system
+    ("held", 64, 4, "half"),             # a cluster, rows split unevenly
+    ("held_float", 90, 7, "float"),      # odd sizes, ragged row groups and vectors
+    ("held_double", 40, 3, "double"),    # FP64 sums and scalars
+    ("held_limit", 160, 8, "half"),      # near the largest that shared memory holds
+    ("streamed", 200, 10, "half"),       # a cluster, rows of G^ streamed
+    ("loop", 256, 16, "half"),           # beyond a cluster: the launch-per-step loop
+])
+def test_reduced_solve_paths(name, N_, p, form):
+    """The reduced solve meets tol_in on the stored G^ for every size class.  The residual
+    is formed in FP64 from the stored blocks; rounding z^ to FP32 adds about 1e-7 to
+    the 1e-5 that the iteration stops at, so 1.1e-5 bounds it."""
+    opts = {"half": dict(factor_prec=N.DDPS_FP32, spike_prec=N.DDPS_BF16X3, ghat_prec=N.DDPS_FP16,
+                         inner_prec=N.DDPS_FP32),
+            "float": dict(factor_prec=N.DDPS_FP32, spike_prec=N.DDPS_FP32, ghat_prec=N.DDPS_FP32,
+                          inner_prec=N.DDPS_FP64),
+            "double": FP64}[form]
+    P = W.small_convdiff_2d(N_, p, seed=N_)
+    S = make_solver(P, tol_in=1e-5, maxit_in=300, **opts)
+    rng = np.random.default_rng(N_)
+    for scale in (1.0, 1e-25, 0.0):  # the scaled copy: squares below FP32's range
+        g = scale * rng.uniform(-1, 1, S.m)
+        z = host(S.reduced_solve(dev(g)))
+        r = g - z
+        for b in range(p):
+            q0, q1, cols = S.ghat_layout(b)
+            r[q0:q1] -= S.ghat_block(b) @ z[cols]
+        assert np.linalg.norm(r) <= 1.1e-5 * np.linalg.norm(g), (name, scale)
