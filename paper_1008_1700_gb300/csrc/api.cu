@@ -13,6 +13,7 @@
 #include <cstring>
 #include <exception>
 #include <fstream>
+#include <future>
 #include <map>
 #include <mutex>
 #include <sstream>
@@ -236,6 +237,15 @@ struct ddps_handle {
   IluDev il{};
   int32_t *il_lf = nullptr, *il_lb = nullptr;
   void* il_val = nullptr;
+  // one-launch block solves: the sweeps in level order per block and their packed
+  // coefficients (il_packed false: the rows' widths differ too much, a launch per level)
+  bool il_packed = false;
+  IluSweep il_l{}, il_u{};
+  int32_t *il_lsrc = nullptr, *il_usrc = nullptr;
+  void *il_lval = nullptr, *il_uval = nullptr;
+  int64_t* block_ptr = nullptr;
+  int64_t il_max_rows = 0;
+  int32_t il_max_level = 0, il_max_starts = 0;
   // launch shape of every block-solve depth and sweep (SOLVE_AUTO until tuned)
   std::vector<int> tune_fwd, tune_bwd;
   std::vector<float> tune_fwd_ms, tune_bwd_ms;
@@ -506,6 +516,11 @@ void factor_launches_ilu(ddps_handle* h, cudaStream_t s) {
                            h->rownorm, h->opt.pivot_tol, h->derr, s);
       h->launches++;
     }
+    if (h->il_packed) {
+      launch_ilu_pack<T>(a, h->il_lsrc, 4 * A.n * h->il_l.groups, (T*)h->il_lval, s);
+      launch_ilu_pack<T>(a, h->il_usrc, 4 * A.n * h->il_u.groups, (T*)h->il_uval, s);
+      h->launches += 2;
+    }
   }
   launch_gather_rt_values(h->vals, h->rt_src, h->nrt, h->rt_val, s);
   h->launches++;
@@ -737,6 +752,12 @@ void block_solve_impl(ddps_handle* h, const double* y, double* g, cudaStream_t s
   if (!u) u = (T*)h->updv;
   const T* arena = (const T*)h->arena;
   Prof pr(h, prof_cls, s);
+  if (A.ilu && h->il_packed) {  // (L~ U~)^-1 y in one launch (the blocks keep their row order)
+    launch_ilu_solve<T>(A.p, h->il_max_rows, h->il_max_level, h->il_max_starts, h->il_l, h->il_u,
+                        (const T*)h->il_lval, (const T*)h->il_uval, A.n, h->block_ptr, y, w, g, s);
+    h->launches++;
+    return;
+  }
   launch_permute_in<T>(y, h->perm, A.n, w, s);
   if (A.ilu) {  // (L~ U~)^-1 y: level-scheduled triangular solves
     const T* a = (const T*)h->il_val;
@@ -1606,6 +1627,81 @@ void build_sparse_forward(ddps_handle* h, const std::vector<int32_t>& kf,
   h->fz = dupload(h, fz);
 }
 
+// The ILU sweeps in level order, block after block (see IluSweep).
+void pack_ilu(ddps_handle* h, int64_t fs) {
+  const Analysis& A = h->A;
+  const int64_t n = A.n;
+  int32_t wl = 0, wu = 0;
+  for (int64_t i = 0; i < n; ++i) {
+    wl = std::max(wl, A.il_diag[i] - A.il_rp[i]);
+    wu = std::max(wu, A.il_rp[i + 1] - A.il_diag[i] - 1);
+  }
+  const int32_t gl = 1 + (std::max(wl - 3, 0) + 3) / 4, gu = 1 + (std::max(wu - 3, 0) + 3) / 4;
+  // every row is padded to the widest: not for patterns with a few long rows
+  if (n * 4 * (int64_t)(gl + gu) > 4 * (int64_t)A.il_col.size() + 16 * n) return;
+  struct Host {
+    std::vector<int32_t> col, src, lev, off, nstarts;
+    int32_t max_level = 0;
+  } lo, up;
+  auto sweep = [&A, n](bool fwd, int32_t groups, Host& H) {
+    const std::vector<int32_t>& list = fwd ? A.il_lf : A.il_lb;
+    const std::vector<int32_t>& lptr = fwd ? A.il_lf_ptr : A.il_lb_ptr;
+    std::vector<int32_t>&col = H.col, &src = H.src, at(A.p, 0), last(A.p, -1);
+    col.assign((size_t)n * 4 * groups, -1);
+    std::vector<std::vector<int32_t>> starts(A.p);  // per block, the starts of its levels
+    src.assign((size_t)n * 4 * groups, -1);
+    for (size_t l = 0; l + 1 < lptr.size(); ++l)
+      for (int32_t q = lptr[l]; q < lptr[l + 1]; ++q) {
+        const int32_t i = list[q], b = A.il_row_block[i], r0 = (int32_t)A.block_ptr[b];
+        const int32_t t = r0 + at[b]++;
+        if (last[b] != (int32_t)l) {  // the block's first row of this level
+          last[b] = (int32_t)l;
+          starts[b].push_back(t);
+        }
+        col[(size_t)t * 4] = i - r0;
+        src[(size_t)t * 4] = A.il_diag[i];
+        const int32_t e0 = fwd ? A.il_rp[i] : A.il_diag[i] + 1, e1 = fwd ? A.il_diag[i] : A.il_rp[i + 1];
+        for (int32_t e = e0; e < e1; ++e) {
+          const int32_t k = e - e0 + 1;
+          const size_t o = ((size_t)(k / 4) * n + t) * 4 + k % 4;
+          col[o] = A.il_col[e] - r0;
+          src[o] = e;
+        }
+      }
+    H.off.assign(1, 0);
+    for (int32_t b = 0; b < A.p; ++b) {
+      starts[b].push_back((int32_t)A.block_ptr[b + 1]);
+      for (size_t l = 0; l + 1 < starts[b].size(); ++l)
+        H.max_level = std::max(H.max_level, starts[b][l + 1] - starts[b][l]);
+      H.nstarts.push_back((int32_t)starts[b].size());
+      H.lev.insert(H.lev.end(), starts[b].begin(), starts[b].end());
+      H.off.push_back((int32_t)H.lev.size());
+    }
+  };
+  // host work only; the future joins the thread and passes on what it throws
+  std::future<void> other = std::async(std::launch::async, [&] { sweep(true, gl, lo); });
+  sweep(false, gu, up);
+  other.get();
+  for (int32_t b = 0; b < A.p; ++b) {
+    h->il_max_starts = std::max(h->il_max_starts, lo.nstarts[b] + up.nstarts[b]);
+    h->il_max_rows = std::max(h->il_max_rows, A.block_ptr[b + 1] - A.block_ptr[b]);
+  }
+  h->il_max_level = std::max(lo.max_level, up.max_level);
+  auto upload = [&](const Host& H, int32_t groups, IluSweep& S) {
+    S.col = dupload(h, H.col);
+    S.lev = dupload(h, H.lev);
+    S.lev_off = dupload(h, H.off);
+    S.groups = groups;
+    return dupload(h, H.src);
+  };
+  h->il_lsrc = upload(lo, gl, h->il_l);
+  h->il_usrc = upload(up, gu, h->il_u);
+  h->il_lval = dalloc_bytes(h, n * 4 * gl * fs);
+  h->il_uval = dalloc_bytes(h, n * 4 * gu * fs);
+  h->block_ptr = dupload(h, A.block_ptr);
+  h->il_packed = true;
+}
+
 void build_device(ddps_handle* h, const int32_t* rowptr, const int32_t* colind) {
   Analysis& A = h->A;
   const int64_t n = A.n, m = (int64_t)A.c.size();
@@ -1655,6 +1751,7 @@ void build_device(ddps_handle* h, const int32_t* rowptr, const int32_t* colind) 
     h->il_lf = dupload(h, A.il_lf);
     h->il_lb = dupload(h, A.il_lb);
     h->il_val = dalloc_bytes(h, std::max<int64_t>((int64_t)A.il_col.size(), 1) * (int64_t)fs);
+    pack_ilu(h, (int64_t)fs);
   }
   CK(cudaMallocHost((void**)&h->herr, 3 * sizeof(long long)));
   // R~

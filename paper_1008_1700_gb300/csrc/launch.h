@@ -89,6 +89,28 @@ struct IluDev {
   const int32_t* diag;
   const int32_t* row_block;
 };
+// One triangular sweep of every block, rows packed in level order (block after
+// block) in `groups` groups of four: col[(q n + t) 4 ..] holds, for row t and q = 0, the
+// local row index and the local columns of the first three entries, for q > 0 the
+// next four (-1: none, at the end); the values are laid out alike, with the diagonal in
+// the row index's place.  Block b's level starts are lev[lev_off[b] ..
+// lev_off[b + 1] - 1].
+struct IluSweep {
+  const int32_t* col;
+  const int32_t* lev;
+  const int32_t* lev_off;
+  int32_t groups;
+};
+// out[i] = a[src[i]], 0 where src[i] < 0
+template <typename T>
+void launch_ilu_pack(const T* a, const int32_t* src, int64_t cnt, T* out, cudaStream_t s);
+// g = (L~ U~)^-1 y, both sweeps of all blocks in one launch; w: n entries of work;
+// max_rows, max_level, max_starts: the largest block, level, and number of level
+// starts of a block's two sweeps
+template <typename T>
+void launch_ilu_solve(int32_t nblocks, int64_t max_rows, int32_t max_level, int32_t max_starts,
+                      const IluSweep& L, const IluSweep& U, const T* lval, const T* uval, int64_t n,
+                      const int64_t* block_ptr, const double* y, T* w, double* g, cudaStream_t s);
 template <typename T>
 void launch_ilu0_level(const int32_t* rows, int32_t nrows, const IluDev& L, T* a,
                        const double* rownorm, double pivot_tol, long long* err, cudaStream_t s);

@@ -91,3 +91,19 @@ def test_ilu_rejects_a_missing_diagonal():
     rowptr = np.concatenate([[0], np.cumsum(counts)]).astype(np.int32)
     with pytest.raises(N.DDPSError, match="INVALID_ARG.*diagonal"):
         Solver(rowptr, colind, P.block_ptr, **ILU64)
+
+
+@pytest.mark.parametrize("name,make", [
+    ("vector_beyond_shared_memory", lambda: W.small_convdiff_2d(180, 1)),  # 32,400 FP64 rows a block
+    ("levels_beyond_the_threads", lambda: W.small_random_dd(6001, 3, k_off=1, seed=4)),
+    ("single_rows", lambda: W.small_random_dd(9, 9, k_off=2, seed=5)),      # blocks of one row
+])
+def test_ilu_one_launch_solves(name, make):
+    """The one-launch block solve where its shapes change; FP64 triangular solves in
+    the oracle's entry order agree to rounding (the bound of the small cases)."""
+    P = make()
+    o = DDPSOracle(P.n, P.rowptr, P.colind, P.values, P.block_ptr, factor="ilu0")
+    y = np.random.default_rng(3).standard_normal(P.n)
+    S = make_solver(P, **ILU64)
+    assert relerr(host(S.block_solve(dev(y))), o.block_solve(y)) <= 1e-12
+    S.close()
