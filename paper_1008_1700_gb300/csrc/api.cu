@@ -558,7 +558,7 @@ void factor_launches_ilu(ddps_handle* h, cudaStream_t s) {
   }
   if (h->use_direct) {
     Prof pr(h, DDPS_PROF_DIRECT_FACTOR, s);
-    h->launches += direct_factor<TG>(h->direct, (const TG*)h->ghat, s);
+    h->launches += direct_factor<TG>(h->direct, (const TG*)h->ghat, h->derr, s);
   }
   check_launch();
 }
@@ -705,7 +705,7 @@ void factor_launches(ddps_handle* h, cudaStream_t s) {
   }
   if (h->use_direct) {
     Prof pr(h, DDPS_PROF_DIRECT_FACTOR, s);
-    h->launches += direct_factor<TG>(h->direct, (const TG*)h->ghat, s);
+    h->launches += direct_factor<TG>(h->direct, (const TG*)h->ghat, h->derr, s);
   }
   check_launch();
 }
@@ -725,7 +725,7 @@ void factor_impl(ddps_handle* h, cudaStream_t s) {
   CK(cudaMemcpyAsync(h->herr, h->derr, 3 * sizeof(long long), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   if (h->herr[0] == 2)
-    throw Fail{DDPS_ERR_TIMEOUT, "a bounded wait of the tensor-core spike products gave up"};
+    throw Fail{DDPS_ERR_TIMEOUT, "a bounded wait of the tensor-core products gave up"};
   if (h->herr[0] != 0) {
     const int64_t row_new = h->herr[2];
     const int64_t row_old = h->A.perm[row_new];

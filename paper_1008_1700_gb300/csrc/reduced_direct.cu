@@ -34,13 +34,7 @@ namespace ddps {
 
 namespace {
 
-// ---------------------------------------------------------------------------
-// Grouped FP32 GEMM: C = alpha A B + beta C, row-major, one launch over the
-// tiles of many problems.  128 x 128 tiles, K in steps of 16 through a double
-// buffer in shared memory, 256 threads each holding an 8 x 8 block of C.
-// ---------------------------------------------------------------------------
-constexpr int GB_M = 128, GB_N = 128, GB_K = 16, GB_T = 256, GB_PAD = 4;
-
+// problem of block t of a grouped launch
 __device__ __forceinline__ int find_problem(const int32_t* __restrict__ prefix, int n, int t) {
   int lo = 0, hi = n;  // prefix[lo] <= t < prefix[hi]
   while (hi - lo > 1) {
@@ -48,91 +42,6 @@ __device__ __forceinline__ int find_problem(const int32_t* __restrict__ prefix, 
     if (prefix[mid] <= t) lo = mid; else hi = mid;
   }
   return lo;
-}
-
-__global__ void __launch_bounds__(GB_T, 2)
-    k_gemm_grouped(const GemmDesc* __restrict__ D, const int32_t* __restrict__ prefix, int32_t np) {
-  __shared__ __align__(16) float As[2][GB_K][GB_M + GB_PAD];
-  __shared__ __align__(16) float Bs[2][GB_K][GB_N + GB_PAD];
-  const int p = find_problem(prefix, np, blockIdx.x);
-  const GemmDesc d = D[p];
-  const int t = blockIdx.x - prefix[p];
-  const int tiles_n = (d.N + GB_N - 1) / GB_N;
-  const int m0 = (t / tiles_n) * GB_M, n0 = (t % tiles_n) * GB_N;
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  // loaders: A 128 x 16 (thread: row tid/2, eight k from (tid&1)*8), B 16 x 128 (rows tid/32 and
-  // tid/32 + 8, four columns each)
-  const int ar = tid >> 1, ak = (tid & 1) * 8;
-  const int bk = tid >> 5, bc = (tid & 31) * 4;
-  float ra[8], rb[8];
-  auto gload = [&](int k0) {
-    const int gr = m0 + ar;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int gk = k0 + ak + q;
-      ra[q] = (gr < d.M && gk < d.K) ? d.A[(int64_t)gr * d.lda + gk] : 0.f;
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int gk = k0 + bk + 8 * h;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int gc = n0 + bc + q;
-        rb[4 * h + q] = (gk < d.K && gc < d.N) ? d.B[(int64_t)gk * d.ldb + gc] : 0.f;
-      }
-    }
-  };
-  auto sstore = [&](int st) {
-#pragma unroll
-    for (int q = 0; q < 8; ++q) As[st][ak + q][ar] = ra[q];
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-      *reinterpret_cast<float4*>(&Bs[st][bk + 8 * h][bc]) =
-          make_float4(rb[4 * h], rb[4 * h + 1], rb[4 * h + 2], rb[4 * h + 3]);
-  };
-  float acc[8][8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
-  const int nk = (d.K + GB_K - 1) / GB_K;
-  if (nk > 0) {
-    gload(0);
-    sstore(0);
-  }
-  __syncthreads();
-  for (int kt = 0; kt < nk; ++kt) {
-    const int st = kt & 1;
-    if (kt + 1 < nk) gload((kt + 1) * GB_K);
-#pragma unroll
-    for (int k = 0; k < GB_K; ++k) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[st][k][ty * 4]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&As[st][k][64 + ty * 4]);
-      const float4 b0 = *reinterpret_cast<const float4*>(&Bs[st][k][tx * 4]);
-      const float4 b1 = *reinterpret_cast<const float4*>(&Bs[st][k][64 + tx * 4]);
-      const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-    }
-    if (kt + 1 < nk) sstore(st ^ 1);
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int r = m0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + (i - 4));
-    if (r >= d.M) continue;
-    float* __restrict__ Cr = d.C + (int64_t)r * d.ldc;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int c = n0 + (j < 4 ? tx * 4 + j : 64 + tx * 4 + (j - 4));
-      if (c >= d.N) continue;
-      const float v = d.alpha * acc[i][j];
-      Cr[c] = d.beta == 0.f ? v : fmaf(d.beta, Cr[c], v);
-    }
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -178,17 +87,23 @@ __global__ void __launch_bounds__(256)
 
 // ---------------------------------------------------------------------------
 // Blocked Gauss-Jordan inversion (no pivoting), one block column kb of
-// width nb per step, for many matrices W (n x n, row-major, ld n):
-//   prep:  Dinv = W(k,k)^-1 (shared memory, one CTA per matrix), Ccol = W(:,k)
-//          with its rows k zeroed, W(i,k) = 0 for i outside k;
-//   GEMM:  Rrow = Dinv W(k,:);
-//   fix:   Rrow(:,k) = Dinv, W(k,:) = Rrow;
-//   GEMM:  W -= Ccol Rrow.
+// width nb = 64 per step, for many matrices W (n x n, row-major, ld n):
+//   prep: Dinv = W(k,k)^-1 (registers, one CTA per matrix), Ccol = W(:,k)
+//         with its rows k zeroed, W(i,k) = 0 for i outside k;
+//   row:  Rrow = Dinv W(k,:) with Rrow(:,k) = Dinv, W(k,:) = Rrow;
+//   GEMM: W -= Ccol Rrow.
+// The steps are a chain, so the small launches count: the 64 x 64 inversion by 256
+// threads with a 4 x 4 block each in registers takes one barrier per pivot; in shared
+// memory with three it made prep 161 us a step (now 12), half of the factorisation.  The panel
+// in 32 rows per CTA, all loads at once: 256 rows in a loop took 30 us.
 // ---------------------------------------------------------------------------
+constexpr int kGjRows = 32;  // rows of the panel per CTA
+
 __global__ void __launch_bounds__(256)
     k_gj_prep(const GjDesc* __restrict__ D, const int32_t* __restrict__ prefix, int32_t np,
-              int32_t kb, int32_t nb) {
-  extern __shared__ float sd[];  // nb x nb
+              int32_t kb) {
+  constexpr int nb = kGjBlock;
+  __shared__ __align__(16) float prow[2][nb], pcol[2][nb];
   const int p = find_problem(prefix, np, blockIdx.x);
   const GjDesc d = D[p];
   const int chunk = blockIdx.x - prefix[p];
@@ -196,63 +111,111 @@ __global__ void __launch_bounds__(256)
   if (kw <= 0) return;
   const int tid = threadIdx.x;
   if (chunk == 0) {
-    for (int e = tid; e < kw * kw; e += blockDim.x) {
-      const int i = e / kw, j = e - i * kw;
-      sd[i * nb + j] = d.W[(int64_t)(k0 + i) * d.n + k0 + j];
-    }
-    __syncthreads();
-    // in-place Gauss-Jordan of the kw x kw block
-    for (int q = 0; q < kw; ++q) {
-      const float piv = 1.f / sd[q * nb + q];
-      __syncthreads();
-      for (int e = tid; e < kw * kw; e += blockDim.x) {
-        const int i = e / kw, j = e - i * kw;
-        if (i == q || j == q) continue;
-        sd[i * nb + j] -= sd[i * nb + q] * piv * sd[q * nb + j];
+    // in-place Gauss-Jordan of the block (identity beyond kw)
+    const int i0 = (tid >> 4) * 4, j0 = (tid & 15) * 4;
+    float a[4][4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const int i = i0 + u, j = j0 + v;
+        a[u][v] = i < kw && j < kw ? d.W[(int64_t)(k0 + i) * d.n + k0 + j] : (i == j ? 1.f : 0.f);
       }
-      __syncthreads();
-      for (int j = tid; j < kw; j += blockDim.x)
-        if (j != q) sd[q * nb + j] *= piv;
-      for (int i = tid; i < kw; i += blockDim.x)
-        if (i != q) sd[i * nb + q] *= -piv;
-      if (tid == 0) sd[q * nb + q] = piv;
-      __syncthreads();
+    for (int q4 = 0; q4 < nb; q4 += 4) {
+      if (q4 >= kw) break;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int q = q4 + r, buf = r & 1;
+        if (i0 == q4) *reinterpret_cast<float4*>(&prow[buf][j0]) = make_float4(a[r][0], a[r][1], a[r][2], a[r][3]);
+        if (j0 == q4) *reinterpret_cast<float4*>(&pcol[buf][i0]) = make_float4(a[0][r], a[1][r], a[2][r], a[3][r]);
+        __syncthreads();
+        const float piv = 1.f / prow[buf][q];
+        const float4 rq = *reinterpret_cast<const float4*>(&prow[buf][j0]);
+        const float4 cq = *reinterpret_cast<const float4*>(&pcol[buf][i0]);
+        const float rv[4] = {rq.x, rq.y, rq.z, rq.w}, cv[4] = {cq.x, cq.y, cq.z, cq.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float cp = cv[u] * piv;
+#pragma unroll
+          for (int v = 0; v < 4; ++v) a[u][v] = a[u][v] - cp * rv[v];
+        }
+        if (i0 == q4)  // the pivot row, then its column
+#pragma unroll
+          for (int v = 0; v < 4; ++v) a[r][v] = rv[v] * piv;
+        if (j0 == q4)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) a[u][r] = i0 + u == q ? piv : cv[u] * -piv;
+      }
     }
-    for (int e = tid; e < kw * kw; e += blockDim.x) {
-      const int i = e / kw, j = e - i * kw;
-      d.Dinv[i * nb + j] = sd[i * nb + j];
-    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int v = 0; v < 4; ++v)
+        if (i0 + u < kw && j0 + v < kw) d.Dinv[(i0 + u) * nb + j0 + v] = a[u][v];
+    return;
   }
-  // column panel, 256 rows per chunk
-  const int r0 = chunk * 256, r1 = min(d.n, r0 + 256);
-  for (int e = tid; e < (r1 - r0) * kw; e += blockDim.x) {
-    const int i = r0 + e / kw, j = e % kw;
-    float* w = d.W + (int64_t)i * d.n + k0 + j;
+  // column panel, kGjRows rows per chunk, all of a thread's loads issued at once
+  const int r0 = (chunk - 1) * kGjRows, j = tid % nb;
+  if (j >= kw) return;
+  constexpr int kPer = kGjRows * nb / 256;
+  float v[kPer];
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    const int i = r0 + tid / nb + u * (256 / nb);
+    v[u] = i < d.n ? d.W[(int64_t)i * d.n + k0 + j] : 0.f;
+  }
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    const int i = r0 + tid / nb + u * (256 / nb);
+    if (i >= d.n) continue;
     const bool in_k = i >= k0 && i < k0 + kw;
-    d.Ccol[(int64_t)i * nb + j] = in_k ? 0.f : *w;
-    if (!in_k) *w = 0.f;
+    d.Ccol[(int64_t)i * nb + j] = in_k ? 0.f : v[u];
+    if (!in_k) d.W[(int64_t)i * d.n + k0 + j] = 0.f;
   }
 }
 
+// Rrow = Dinv W(k,:) for 64 columns per CTA (Dinv and the 64 rows in shared memory, 4 x 4
+// results per thread), written to Rrow and back to W(k,:).
 __global__ void __launch_bounds__(256)
-    k_gj_fix(const GjDesc* __restrict__ D, const int32_t* __restrict__ prefix, int32_t np,
-             int32_t kb, int32_t nb) {
+    k_gj_row(const GjDesc* __restrict__ D, const int32_t* __restrict__ prefix, int32_t np,
+             int32_t kb) {
+  constexpr int nb = kGjBlock;
+  __shared__ __align__(16) float Ds[nb][nb + 4], Ws[nb][nb + 4];  // Ds transposed
   const int p = find_problem(prefix, np, blockIdx.x);
   const GjDesc d = D[p];
+  const int c0 = (blockIdx.x - prefix[p]) * nb;
   const int k0 = kb * nb, kw = min(nb, d.n - k0);
   if (kw <= 0) return;
-  const int chunk = blockIdx.x - prefix[p];
-  const int64_t total = (int64_t)kw * d.n;
-  for (int64_t e = (int64_t)chunk * 2048 + threadIdx.x; e < min(total, (int64_t)(chunk + 1) * 2048);
-       e += blockDim.x) {
-    const int i = (int)(e / d.n), j = (int)(e - (int64_t)i * d.n);
-    float v = d.Rrow[(int64_t)i * d.n + j];
-    if (j >= k0 && j < k0 + kw) {
-      v = d.Dinv[i * nb + (j - k0)];
-      d.Rrow[(int64_t)i * d.n + j] = v;
-    }
-    d.W[(int64_t)(k0 + i) * d.n + j] = v;
+  const int tid = threadIdx.x;
+#pragma unroll 8
+  for (int e = tid; e < nb * nb; e += 256) {
+    const int i = e / nb, j = e % nb;
+    Ds[j][i] = i < kw && j < kw ? d.Dinv[i * nb + j] : 0.f;
+    Ws[i][j] = i < kw && c0 + j < d.n ? d.W[(int64_t)(k0 + i) * d.n + c0 + j] : 0.f;
   }
+  __syncthreads();
+  const int i0 = (tid >> 4) * 4, j0 = (tid & 15) * 4;
+  float acc[4][4] = {};
+#pragma unroll 8
+  for (int k = 0; k < nb; ++k) {
+    const float4 a = *reinterpret_cast<const float4*>(&Ds[k][i0]);
+    const float4 b = *reinterpret_cast<const float4*>(&Ws[k][j0]);
+    const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(av[u], bv[v], acc[u][v]);
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const int i = i0 + u, j = c0 + j0 + v;
+      if (i >= kw || j >= d.n) continue;
+      const float r = j >= k0 && j < k0 + kw ? Ds[j - k0][i] : acc[u][v];
+      d.Rrow[(int64_t)i * d.n + j] = r;
+      d.W[(int64_t)(k0 + i) * d.n + j] = r;
+    }
 }
 
 // Writes M = I - E(0:nj, :) (the rows J of E) into W and copies the rows J'
@@ -332,10 +295,10 @@ GroupLaunch<Desc> dev(const Desc* base, const int32_t* prefix, const GroupLaunch
 // ---------------------------------------------------------------------------
 namespace {
 
-int64_t run_gemm(const DirectPlan& P, const GroupLaunchHost& L, cudaStream_t s) {
+int64_t run_gemm(const DirectPlan& P, const GroupLaunchHost& L, long long* err, cudaStream_t s) {
   if (L.nblocks <= 0) return 0;
   const GroupLaunch<GemmDesc> g = dev(P.d_gemm, P.d_prefix, L);
-  k_gemm_grouped<<<g.nblocks, GB_T, 0, s>>>(g.desc, g.prefix, g.np);
+  launch_gemm_grouped_tc(g.desc, g.prefix, g.np, g.nblocks, err, s);
   return 1;
 }
 int64_t run_gemv(const DirectPlan& P, const GroupLaunchHost& L, cudaStream_t s) {
@@ -366,7 +329,7 @@ int64_t run_form(const DirectPlan& P, const GroupLaunchHost& L, cudaStream_t s) 
 }  // namespace
 
 template <typename TG>
-int64_t direct_factor(const DirectPlan& P, const TG* ghat, cudaStream_t s) {
+int64_t direct_factor(const DirectPlan& P, const TG* ghat, long long* err, cudaStream_t s) {
   int64_t n = 0;
   for (const GroupLaunchHost& L : P.extract) {
     if (L.nblocks <= 0) continue;
@@ -374,39 +337,31 @@ int64_t direct_factor(const DirectPlan& P, const TG* ghat, cudaStream_t s) {
     k_extract_lu<TG><<<g.nblocks, 256, 0, s>>>(g.desc, g.prefix, g.np, ghat);
     ++n;
   }
-  const size_t gj_sm = (size_t)kGjBlock * kGjBlock * sizeof(float);
-  if (gj_sm > 48 * 1024)
-    record_launch_error(
-        cudaFuncSetAttribute(k_gj_prep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gj_sm));
   for (int32_t t = 1; t < P.nsteps; ++t) {
     const DirectPlan::FactorStep& st = P.fstep[t];
     n += run_copy(P, st.copy, s);
-    n += run_gemm(P, st.gemm_y, s);
-    n += run_gemm(P, st.gemm_k, s);
+    n += run_gemm(P, st.gemm_y, err, s);
+    n += run_gemm(P, st.gemm_k, err, s);
     n += run_gather(P, st.gather_q, s);
-    n += run_gemm(P, st.gemm_e, s);
+    n += run_gemm(P, st.gemm_e, err, s);
     n += run_form(P, st.form, s);
     for (int32_t kb = 0; kb < st.kb; ++kb) {
       if (st.gj_prep.nblocks > 0) {
         const GroupLaunch<GjDesc> g = dev(P.d_gj, P.d_prefix, st.gj_prep);
-        k_gj_prep<<<g.nblocks, 256, gj_sm, s>>>(g.desc, g.prefix, g.np, kb, kGjBlock);
-        ++n;
+        k_gj_prep<<<g.nblocks, 256, 0, s>>>(g.desc, g.prefix, g.np, kb);
+        const GroupLaunch<GjDesc> r = dev(P.d_gj, P.d_prefix, st.gj_row);
+        k_gj_row<<<r.nblocks, 256, 0, s>>>(r.desc, r.prefix, r.np, kb);
+        n += 2;
       }
-      n += run_gemm(P, st.gj_rrow[kb], s);
-      if (st.gj_fix.nblocks > 0) {
-        const GroupLaunch<GjDesc> g = dev(P.d_gj, P.d_prefix, st.gj_fix);
-        k_gj_fix<<<g.nblocks, 256, 0, s>>>(g.desc, g.prefix, g.np, kb, kGjBlock);
-        ++n;
-      }
-      n += run_gemm(P, st.gj_update[kb], s);
+      n += run_gemm(P, st.gj_update[kb], err, s);
     }
   }
   return n;
 }
-template int64_t direct_factor<double>(const DirectPlan&, const double*, cudaStream_t);
-template int64_t direct_factor<float>(const DirectPlan&, const float*, cudaStream_t);
-template int64_t direct_factor<__half>(const DirectPlan&, const __half*, cudaStream_t);
-template int64_t direct_factor<__nv_bfloat16>(const DirectPlan&, const __nv_bfloat16*, cudaStream_t);
+template int64_t direct_factor<double>(const DirectPlan&, const double*, long long*, cudaStream_t);
+template int64_t direct_factor<float>(const DirectPlan&, const float*, long long*, cudaStream_t);
+template int64_t direct_factor<__half>(const DirectPlan&, const __half*, long long*, cudaStream_t);
+template int64_t direct_factor<__nv_bfloat16>(const DirectPlan&, const __nv_bfloat16*, long long*, cudaStream_t);
 
 int64_t direct_solve(const DirectPlan& P, const double* ghat_in, double* zhat_out, cudaStream_t s) {
   if (P.m <= 0) return 0;
@@ -474,7 +429,7 @@ static GroupLaunchHost add_launch(std::vector<Desc>& all_desc, std::vector<int32
 
 static int32_t gemm_tiles(int M, int N) {
   if (M <= 0 || N <= 0) return 0;
-  return ((M + GB_M - 1) / GB_M) * ((N + GB_N - 1) / GB_N);
+  return ((M + 127) / 128) * ((N + 127) / 128);
 }
 static int32_t chunks_2048(int64_t count) { return (int32_t)((count + 2047) / 2048); }
 
@@ -641,14 +596,14 @@ std::string plan_direct(const DirectInput& in, DirectPlan& P, const DeviceAlloc&
     DirectPlan::FactorStep& st = P.fstep[t];
     std::vector<CopyDesc> cp;
     std::vector<int32_t> cpn;
-    std::vector<GemmDesc> g1, g2, g3, gr, gu;
+    std::vector<GemmDesc> g1, g2, g3;
     std::vector<int32_t> g1n, g2n, g3n;
     std::vector<GatherDesc> ga;
     std::vector<int32_t> gan;
     std::vector<FormDesc> fm;
     std::vector<int32_t> fmn;
     std::vector<GjDesc> gj;
-    std::vector<int32_t> gjn_prep, gjn_fix;
+    std::vector<int32_t> gjn_prep, gjn_row;
     int32_t kb_max = 0;
     for (int32_t b = 0; b < p; ++b) {
       if (tpos[b] != t) continue;
@@ -684,8 +639,8 @@ std::string plan_direct(const DirectInput& in, DirectPlan& P, const DeviceAlloc&
         fm.push_back(FormDesc{E, F(offW[b]), F(offC[b]), sb, na});
         fmn.push_back(chunks_2048((int64_t)sb * na));
         gj.push_back(GjDesc{F(offW[b]), P.ebuf + offR[b], P.ebuf + offCc[b], P.ebuf + offD[b], na});
-        gjn_prep.push_back((na + 255) / 256);
-        gjn_fix.push_back(chunks_2048((int64_t)kGjBlock * na));
+        gjn_prep.push_back(1 + (na + kGjRows - 1) / kGjRows);
+        gjn_row.push_back((na + kGjBlock - 1) / kGjBlock);
         kb_max = std::max(kb_max, (na + kGjBlock - 1) / kGjBlock);
         (void)sa;
       }
@@ -697,23 +652,19 @@ std::string plan_direct(const DirectInput& in, DirectPlan& P, const DeviceAlloc&
     st.gemm_e = add_launch(P.gemm_desc, P.prefix, g3, g3n);
     st.form = add_launch(P.form_desc, P.prefix, fm, fmn);
     st.gj_prep = add_launch(P.gj_desc, P.prefix, gj, gjn_prep);
-    st.gj_fix = add_launch(P.gj_desc, P.prefix, gj, gjn_fix);
-    // Gauss-Jordan GEMMs per column block kb: Rrow = Dinv W(k,:), W -= Ccol Rrow
+    st.gj_row = add_launch(P.gj_desc, P.prefix, gj, gjn_row);
+    // the Gauss-Jordan GEMM per column block kb: W -= Ccol Rrow
     for (int32_t kb = 0; kb < kb_max; ++kb) {
-      std::vector<GemmDesc> r1, r2;
-      std::vector<int32_t> r1n, r2n;
+      std::vector<GemmDesc> r2;
+      std::vector<int32_t> r2n;
       for (const GjDesc& q : gj) {
         const int32_t k0 = kb * kGjBlock, kw = std::min(kGjBlock, q.n - k0);
         if (kw <= 0) {
           continue;
         }
-        r1.push_back(GemmDesc{q.Dinv, q.W + (int64_t)k0 * q.n, q.Rrow, kw, q.n, kw, kGjBlock, q.n,
-                              q.n, 1.f, 0.f});
-        r1n.push_back(gemm_tiles(kw, q.n));
         r2.push_back(GemmDesc{q.Ccol, q.Rrow, q.W, q.n, q.n, kw, kGjBlock, q.n, q.n, -1.f, 1.f});
         r2n.push_back(gemm_tiles(q.n, q.n));
       }
-      st.gj_rrow.push_back(add_launch(P.gemm_desc, P.prefix, r1, r1n));
       st.gj_update.push_back(add_launch(P.gemm_desc, P.prefix, r2, r2n));
     }
     st.kb = kb_max;

@@ -125,8 +125,8 @@ struct DirectPlan {
   int32_t* d_prefix = nullptr;
   std::vector<GroupLaunchHost> extract;
   struct FactorStep {
-    GroupLaunchHost copy, gemm_y, gemm_k, gather_q, gemm_e, form, gj_prep, gj_fix;
-    std::vector<GroupLaunchHost> gj_rrow, gj_update;
+    GroupLaunchHost copy, gemm_y, gemm_k, gather_q, gemm_e, form, gj_prep, gj_row;
+    std::vector<GroupLaunchHost> gj_update;
     int32_t kb = 0;
   };
   std::vector<FactorStep> fstep;
@@ -143,8 +143,12 @@ std::string plan_direct(const DirectInput& in, DirectPlan& P, const DeviceAlloc&
 void upload_direct(DirectPlan& P, const DeviceAlloc& alloc);
 // Factor: L_b, U_b from the stored G^ (element type TG), then W_b, C_b in
 // chain order.  Returns the number of launches.
+// A wait of the tensor-core products that runs out writes 2 into err[0].
 template <typename TG>
-int64_t direct_factor(const DirectPlan& P, const TG* ghat, cudaStream_t s);
+int64_t direct_factor(const DirectPlan& P, const TG* ghat, long long* err, cudaStream_t s);
+// spike_tc.cu: the GEMMs of one grouped launch (128 x 128 tiles) on the tensor cores
+void launch_gemm_grouped_tc(const GemmDesc* desc, const int32_t* prefix, int32_t np, int32_t nblocks,
+                            long long* err, cudaStream_t s);
 // z^ = G^-1 g^ (device FP64 vectors of m entries in c order).  Returns the
 // number of launches.
 int64_t direct_solve(const DirectPlan& P, const double* ghat_in, double* zhat_out, cudaStream_t s);

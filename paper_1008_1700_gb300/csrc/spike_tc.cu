@@ -25,6 +25,7 @@
 #include <cstdint>
 
 #include "launch.h"
+#include "reduced_direct.h"
 
 namespace ddps {
 
@@ -567,6 +568,245 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                  "r"((uint32_t)TC_BN));
+}
+
+// ---------------------------------------------------------------------------
+// Grouped FP32 GEMM on the tensor cores, C = alpha A B + beta C (row-major), for the
+// block LU of the reduced system: one launch over the 128 x 128 tiles of many
+// problems.  Every operand is split into three bf16 parts (x = h + m + l, 24 bits, the
+// FP32 significand) and the six products of order 2^-16 and above are taken: h h, h m,
+// m h, m m, h l, l h; what is left out is below 2^-24 of a term, an FP32 rounding.
+// The tensor core adds to its accumulator with truncation, so h h has an accumulator of
+// its own (the other products, 2^-8 of it and less, share a second one) and a sum stays
+// there for 32 values of K only, then it is added to FP32 registers: the reduced solves
+// are as exact as with FP32 FMAs (residuals within 10% either way on six grids; with one
+// accumulator and 256 values those of 2-D grids were three times as large).
+// The 256 threads load and split the next 32 values of K while the MMAs of the last
+// ones run (two stages).  Bound by the splitting and the MMAs
+// (about 800 and 880 cycles per 32 values of K and tile): 4608 x 2304 x 2304 takes
+// 508 us (96 TFLOP/s of the product) against 1,321 on the FP32 cores, the rank-64 update
+// of a 2304 x 2304 block 19.6 us against 50.7 (38 before C went through shared memory).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void split3(const float* v, unsigned char* h, unsigned char* m,
+                                       unsigned char* l) {
+  uint32_t a[4], b[4], c[4];
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    a[t] = cvt_bf16x2(v[2 * t], v[2 * t + 1]);
+    const float r0 = v[2 * t] - __uint_as_float(a[t] << 16);
+    const float r1 = v[2 * t + 1] - __uint_as_float(a[t] & 0xffff0000u);
+    b[t] = cvt_bf16x2(r0, r1);
+    c[t] = cvt_bf16x2(r0 - __uint_as_float(b[t] << 16), r1 - __uint_as_float(b[t] & 0xffff0000u));
+  }
+  *reinterpret_cast<uint4*>(h) = make_uint4(a[0], a[1], a[2], a[3]);
+  *reinterpret_cast<uint4*>(m) = make_uint4(b[0], b[1], b[2], b[3]);
+  *reinterpret_cast<uint4*>(l) = make_uint4(c[0], c[1], c[2], c[3]);
+}
+
+constexpr int GG_GROUP = 1;  // stages of 32 per tensor-memory sum
+constexpr uint32_t GG_STAGE = 6 * TC_TILE_BYTES;
+
+__global__ void __launch_bounds__(TC_THREADS, 2)
+    k_gemm_grouped_tc(const GemmDesc* __restrict__ D, const int32_t* __restrict__ prefix,
+                      int32_t np, long long* __restrict__ err) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ __align__(8) uint64_t empty[2];
+  __shared__ uint32_t tmem_slot;
+  int lo = 0, hi = np;  // prefix[lo] <= blockIdx.x < prefix[hi]
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (prefix[mid] <= (int)blockIdx.x) lo = mid; else hi = mid;
+  }
+  const GemmDesc d = D[lo];
+  const int t = blockIdx.x - prefix[lo];
+  const int tiles_n = (d.N + TC_BN - 1) / TC_BN;
+  const int m0 = (t / tiles_n) * TC_BM, n0 = (t % tiles_n) * TC_BN;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(&tmem_slot)),
+                 "r"((uint32_t)(2 * TC_BN)));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  if (tid == 0) {
+    for (int i = 0; i < 2; ++i)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&empty[i])));
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tmem_slot;
+  const uint32_t sbase = smem_u32(smem);
+  bool timed_out = false;
+
+  // A: rows of K-contiguous values, runs of 8 of one row; B: columns on the lanes
+  const bool vec = d.lda % 4 == 0 && ((uintptr_t)d.A & 15) == 0;
+  float areg[2][8], breg[2][8];
+  auto load = [&](int kt) {
+    const int k0 = kt * TC_BK;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int e = tid + q * TC_THREADS;
+      const int gi = m0 + e / 4, ka = k0 + (e % 4) * 8;
+      const float* __restrict__ a = d.A + (int64_t)gi * d.lda + ka;
+      if (vec && gi < d.M && ka + 8 <= d.K) {
+        const float4 x = *reinterpret_cast<const float4*>(a), y = *reinterpret_cast<const float4*>(a + 4);
+        areg[q][0] = x.x, areg[q][1] = x.y, areg[q][2] = x.z, areg[q][3] = x.w;
+        areg[q][4] = y.x, areg[q][5] = y.y, areg[q][6] = y.z, areg[q][7] = y.w;
+      } else {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) areg[q][u] = gi < d.M && ka + u < d.K ? a[u] : 0.f;
+      }
+      const int gj = n0 + e % TC_BN, kb = k0 + (e / TC_BN) * 8;
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        breg[q][u] = gj < d.N && kb + u < d.K ? d.B[(int64_t)(kb + u) * d.ldb + gj] : 0.f;
+    }
+  };
+  // this thread's part of the tile: row quarter * 32 + lane, columns half * 64 .. + 63
+  const int quarter = warp & 3, half = warp >> 2;
+  float acc[64];
+#pragma unroll
+  for (int u = 0; u < 64; ++u) acc[u] = 0.f;
+  auto collect = [&]() {  // adds the two accumulators (their MMAs have completed)
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+    for (int c = 0; c < 64; c += 16) {
+      float v[16];
+#pragma unroll
+      for (int h = 1; h >= 0; --h) {
+        uint32_t rv[16];
+        const uint32_t taddr = tmem + (uint32_t)(h * TC_BN) + ((uint32_t)(quarter * 32) << 16) +
+                               (uint32_t)(half * 64 + c);
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
+            "%11, %12, %13, %14, %15}, [%16];"
+            : "=r"(rv[0]), "=r"(rv[1]), "=r"(rv[2]), "=r"(rv[3]), "=r"(rv[4]), "=r"(rv[5]),
+              "=r"(rv[6]), "=r"(rv[7]), "=r"(rv[8]), "=r"(rv[9]), "=r"(rv[10]), "=r"(rv[11]),
+              "=r"(rv[12]), "=r"(rv[13]), "=r"(rv[14]), "=r"(rv[15])
+            : "r"(taddr));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int u = 0; u < 16; ++u) v[u] = h ? __uint_as_float(rv[u]) : v[u] + __uint_as_float(rv[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < 16; ++u) acc[c + u] += v[u];
+    }
+    // ordered before the MMAs that refill the accumulators (after the next barrier)
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  };
+
+  const int nk = (d.K + TC_BK - 1) / TC_BK;
+  if (nk > 0) load(0);
+  for (int kt = 0; kt < nk; ++kt) {
+    const int st = kt & 1;
+    if (kt >= 2 && !timed_out)
+      timed_out = !mbar_wait(smem_u32(&empty[st]), ((kt - 2) >> 1) & 1, err);
+    unsigned char* sA = smem + st * GG_STAGE;
+    unsigned char* sB = sA + 3 * TC_TILE_BYTES;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int e = tid + q * TC_THREADS;
+      const uint32_t oa = chunk_off(e / 4, e % 4), ob = chunk_off(e % TC_BN, e / TC_BN);
+      split3(areg[q], sA + oa, sA + TC_TILE_BYTES + oa, sA + 2 * TC_TILE_BYTES + oa);
+      split3(breg[q], sB + ob, sB + TC_TILE_BYTES + ob, sB + 2 * TC_TILE_BYTES + ob);
+    }
+    if (kt + 1 < nk) load(kt + 1);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    const bool first = kt % GG_GROUP == 0;
+    if (first && kt > 0 && !timed_out)
+      timed_out = !mbar_wait(smem_u32(&empty[(kt - 1) & 1]), ((kt - 1) >> 1) & 1, err);
+    timed_out = __syncthreads_or(timed_out);  // all threads give up together
+    if (timed_out) break;
+    if (first && kt > 0) {  // the group before is complete
+      collect();
+      __syncthreads();
+    }
+    if (tid == 0) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t aS = sbase + st * GG_STAGE, bS = aS + 3 * TC_TILE_BYTES;
+      const uint32_t lowp = tmem + TC_BN;
+#pragma unroll
+      for (int kk = 0; kk < TC_BK / 16; ++kk) {
+        const uint32_t ko = kk * 256;
+        uint64_t a[3], b[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          a[q] = make_desc(aS + q * TC_TILE_BYTES + ko, 128, kSBO);
+          b[q] = make_desc(bS + q * TC_TILE_BYTES + ko, 128, kSBO);
+        }
+        const uint32_t more = !first || kk > 0;
+        mma_bf16(lowp, a[2], b[0], more);
+        mma_bf16(lowp, a[0], b[2], 1u);
+        mma_bf16(lowp, a[1], b[1], 1u);
+        mma_bf16(lowp, a[1], b[0], 1u);
+        mma_bf16(lowp, a[0], b[1], 1u);
+        mma_bf16(tmem, a[0], b[0], more);
+      }
+      mma_commit(smem_u32(&empty[st]));
+    }
+  }
+  if (nk > 0 && !timed_out) {
+    timed_out = !mbar_wait(smem_u32(&empty[(nk - 1) & 1]), ((nk - 1) >> 1) & 1, err);
+    timed_out = __syncthreads_or(timed_out);
+    if (!timed_out) collect();
+  }
+  if (timed_out && tid == 0) atomicCAS((unsigned long long*)&err[0], 0ull, 2ull);
+  if (!timed_out) {
+    // the warp's 32 x 64 part is turned around in shared memory (the stages are free), so
+    // that a row's 256 bytes of C are read and written by 16 lanes, eight loads in flight
+    float* tb = reinterpret_cast<float*>(smem) + warp * 32 * 68;
+#pragma unroll
+    for (int c = 0; c < 64; c += 4)
+      *reinterpret_cast<float4*>(tb + lane * 68 + c) =
+          make_float4(d.alpha * acc[c], d.alpha * acc[c + 1], d.alpha * acc[c + 2], d.alpha * acc[c + 3]);
+    __syncwarp();
+    const int cc = (lane & 15) * 4, gc = n0 + half * 64 + cc;
+    const bool cvec = d.ldc % 4 == 0 && ((uintptr_t)d.C & 15) == 0 && gc + 4 <= d.N;
+#pragma unroll
+    for (int r0 = 0; r0 < 32; r0 += 16) {
+      float4 x[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int gi = m0 + quarter * 32 + r0 + 2 * u + (lane >> 4);
+        x[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (d.beta == 0.f || gi >= d.M) continue;
+        const float* __restrict__ C = d.C + (int64_t)gi * d.ldc + gc;
+        if (cvec) {
+          x[u] = *reinterpret_cast<const float4*>(C);
+        } else {
+          if (gc < d.N) x[u].x = C[0];
+          if (gc + 1 < d.N) x[u].y = C[1];
+          if (gc + 2 < d.N) x[u].z = C[2];
+          if (gc + 3 < d.N) x[u].w = C[3];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int row = r0 + 2 * u + (lane >> 4), gi = m0 + quarter * 32 + row;
+        if (gi >= d.M) continue;
+        float4 v = *reinterpret_cast<const float4*>(tb + row * 68 + cc);
+        if (d.beta != 0.f)
+          v = make_float4(fmaf(d.beta, x[u].x, v.x), fmaf(d.beta, x[u].y, v.y),
+                          fmaf(d.beta, x[u].z, v.z), fmaf(d.beta, x[u].w, v.w));
+        float* __restrict__ C = d.C + (int64_t)gi * d.ldc + gc;
+        if (cvec) {
+          *reinterpret_cast<float4*>(C) = v;
+        } else {
+          if (gc < d.N) C[0] = v.x;
+          if (gc + 1 < d.N) C[1] = v.y;
+          if (gc + 2 < d.N) C[2] = v.z;
+          if (gc + 3 < d.N) C[3] = v.w;
+        }
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                 "r"((uint32_t)(2 * TC_BN)));
 }
 
 // ---------------------------------------------------------------------------
@@ -1465,6 +1705,14 @@ void launch_lu_update_tc(DevFronts F, const int32_t* tile_front, const int32_t* 
   const size_t sm = 2 * 4 * (size_t)TC_TILE_BYTES;  // two stages of L and U, high and low parts
   record_launch_error(cudaFuncSetAttribute(k_lu_update_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   k_lu_update_tc<<<ntiles, TC_THREADS, sm, s>>>(F, tile_front, tile_ij, j0, arena, err);
+}
+void launch_gemm_grouped_tc(const GemmDesc* desc, const int32_t* prefix, int32_t np, int32_t nblocks,
+                            long long* err, cudaStream_t s) {
+  if (nblocks <= 0) return;
+  const size_t sm = 2 * (size_t)GG_STAGE;
+  record_launch_error(
+      cudaFuncSetAttribute(k_gemm_grouped_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  k_gemm_grouped_tc<<<nblocks, TC_THREADS, sm, s>>>(desc, prefix, np, err);
 }
 int64_t tc_a_block_bytes(int passes) { return (passes == 3 ? 2 : 1) * (int64_t)TC_TILE_BYTES; }
 

@@ -108,3 +108,24 @@ def test_direct_rejects_partitions_that_are_not_chains():
     with pytest.raises(N.DDPSError, match="INVALID_ARG.*EXPLICIT"):
         Solver(Q.rowptr, Q.colind, Q.block_ptr, ghat_mode=N.DDPS_GHAT_IMPLICIT,
                **{k: v for k, v in FP64_DIRECT.items()})
+
+
+@pytest.mark.parametrize("name,make", [
+    ("one_step", lambda: W.small_convdiff_2d(21, 3)),          # 21 columns: part of a 32-column stage
+    ("two_steps", lambda: W.small_convdiff_2d(97, 4)),         # Gauss-Jordan steps of 64 and 33
+    ("odd_planes", lambda: W.small_convdiff_3d(13, [4, 5, 4])),  # 169 columns, rows not 16-byte aligned
+    ("tiles", lambda: W.small_convdiff_3d(20, [5, 5, 5, 5])),  # 400 columns: ragged 128 x 128 tiles
+])
+def test_block_lu_on_the_stored_matrix(name, make):
+    """The direct reduced solve satisfies the stored G^ in FP64 to FP32 accuracy: the block
+    LU's products of up to 800 terms round to about 1e-6, 1e-5 bounds it."""
+    P = make()
+    S = make_solver(P, **MIXED_DIRECT)
+    g = np.random.default_rng(2).uniform(-1, 1, S.m)
+    z = host(S.reduced_solve(dev(g)))
+    r = g - z
+    for b in range(P.p):
+        q0, q1, cols = S.ghat_layout(b)
+        r[q0:q1] -= S.ghat_block(b) @ z[cols]
+    assert np.linalg.norm(r) <= 1e-5 * np.linalg.norm(g), name
+    S.close()
