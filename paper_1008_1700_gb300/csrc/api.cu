@@ -255,6 +255,7 @@ struct ddps_handle {
   // persistent sweeps of the block solve over the levels >= persist_L (fronts of at
   // most kPersistM rows): orders, waits and flags (2 nfronts done flags, 2 counters)
   int32_t persist_L = -1, persist_n = 0, persist_max_m = 0;
+  bool use_persist = false;  // taken instead of launches per depth (the autotuner times both)
   int32_t *p_fwd = nullptr, *p_bwd = nullptr, *p_wait = nullptr, *p_flags = nullptr;
   // the inner BiCGStab of small systems in one launch (inner.ok false: a system is too large)
   InnerPlan inner;
@@ -264,9 +265,9 @@ struct ddps_handle {
   // CUDA graphs: launch sequences that repeat unchanged are captured once on
   // a stream of the handle and replayed (not while profiling is on)
   cudaStream_t gstream = nullptr;
-  cudaEvent_t gev[2] = {nullptr, nullptr};
-  cudaGraphExec_t g_inner = nullptr, g_factor = nullptr;
-  int64_t g_inner_launches = 0, g_factor_launches = 0;
+  cudaGraphExec_t g_inner = nullptr, g_factor = nullptr, g_sweeps = nullptr;
+  int64_t g_inner_launches = 0, g_factor_launches = 0, g_sweeps_launches = 0;
+  bool capturing = false;  // a capture is under way: launches go into it
   struct PrecGraph {
     const double* y;
     double* z;
@@ -408,16 +409,25 @@ void check_launch() {
 
 // ---------------------------------------------------------------------------
 // CUDA graphs.  A capture runs on the handle's own stream (the legacy default
-// stream cannot be captured); a replay is ordered after the caller's stream
-// and the caller's stream after it, through two events.
+// stream cannot be captured); a replay is launched into the caller's stream.
 // ---------------------------------------------------------------------------
 bool graphs_on(const ddps_handle* h) { return h->opt.use_graphs && h->prof_mask == 0; }
+
+// Whether a sequence that may be called under a capture (the handle's own or the
+// caller's) can be replayed here: under a capture the launches themselves are enqueued.
+bool replays_in(const ddps_handle* h, cudaStream_t s) {
+  if (!graphs_on(h) || h->capturing) return false;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return st == cudaStreamCaptureStatusNone;
+}
 
 void ensure_graph_stream(ddps_handle* h) {
   if (h->gstream) return;
   CK(cudaStreamCreateWithFlags(&h->gstream, cudaStreamNonBlocking));
-  CK(cudaEventCreateWithFlags(&h->gev[0], cudaEventDisableTiming));
-  CK(cudaEventCreateWithFlags(&h->gev[1], cudaEventDisableTiming));
 }
 
 // Captures the launches `body` enqueues on the handle's stream; returns the
@@ -427,9 +437,12 @@ cudaGraphExec_t capture_graph(ddps_handle* h, F body, int64_t* count) {
   ensure_graph_stream(h);
   const int64_t l0 = h->launches;
   CK(cudaStreamBeginCapture(h->gstream, cudaStreamCaptureModeRelaxed));
+  h->capturing = true;
   try {
     body(h->gstream);
+    h->capturing = false;
   } catch (...) {
+    h->capturing = false;
     cudaGraph_t g = nullptr;
     cudaStreamEndCapture(h->gstream, &g);
     if (g) cudaGraphDestroy(g);
@@ -448,11 +461,7 @@ cudaGraphExec_t capture_graph(ddps_handle* h, F body, int64_t* count) {
 }
 
 void replay_graph(ddps_handle* h, cudaGraphExec_t exec, int64_t count, cudaStream_t s) {
-  CK(cudaEventRecord(h->gev[0], s));
-  CK(cudaStreamWaitEvent(h->gstream, h->gev[0], 0));
-  CK(cudaGraphLaunch(exec, h->gstream));
-  CK(cudaEventRecord(h->gev[1], h->gstream));
-  CK(cudaStreamWaitEvent(s, h->gev[1], 0));
+  CK(cudaGraphLaunch(exec, s));
   h->launches += count;
 }
 
@@ -742,6 +751,36 @@ void factor_impl(ddps_handle* h, cudaStream_t s) {
 // ---------------------------------------------------------------------------
 // Fig. 3 step 6.1 (and the second block solve of the retrieval)
 // ---------------------------------------------------------------------------
+// Both sweeps over the permuted vector w (u: the fronts' update vectors): levels >= top one
+// persistent launch per sweep, the levels above one launch each.
+template <typename T>
+void sweep_launches(ddps_handle* h, T* w, T* u, cudaStream_t s) {
+  const Analysis& A = h->A;
+  const T* arena = (const T*)h->arena;
+  const int top = h->use_persist ? h->persist_L : A.nlevels;
+  const int64_t nf = (int64_t)A.f_k.size();
+  int32_t* done_f = h->p_flags;
+  int32_t* done_b = h->p_flags + nf;
+  if (h->use_persist) {
+    CK(cudaMemsetAsync(h->p_flags, 0, (2 * nf + 2) * sizeof(int32_t), s));
+    launch_fwd_persist<T>(h->F, h->p_fwd, h->persist_n, h->persist_max_m, arena, w, u, done_f,
+                          h->p_flags + 2 * nf, h->derr, s);
+    h->launches++;
+  }
+  for (int L = top - 1; L >= 0; --L)
+    launch_fwd1<T>(h->F, h->level_fronts + A.level_ptr[L], A.level_ptr[L + 1] - A.level_ptr[L],
+                   h->split[L].max_m, arena, w, u, s, h->tune_fwd.empty() ? SOLVE_AUTO : h->tune_fwd[L]);
+  for (int L = 0; L < top; ++L)
+    launch_bwd1<T>(h->F, h->level_fronts + A.level_ptr[L], A.level_ptr[L + 1] - A.level_ptr[L],
+                   h->split[L].max_m, arena, w, s, h->tune_bwd.empty() ? SOLVE_AUTO : h->tune_bwd[L]);
+  if (h->use_persist) {
+    launch_bwd_persist<T>(h->F, h->p_bwd, h->persist_n, h->persist_max_m, h->p_wait, arena, w,
+                          done_b, h->p_flags + 2 * nf + 1, h->derr, s);
+    h->launches++;
+  }
+  h->launches += 2 * top;
+}
+
 // w, u: the permuted vector (n entries) and the fronts' update vectors; the
 // handle's workspace unless the caller passes its own scratch.
 template <typename T>
@@ -750,7 +789,6 @@ void block_solve_impl(ddps_handle* h, const double* y, double* g, cudaStream_t s
   const Analysis& A = h->A;
   if (!w) w = (T*)h->w;
   if (!u) u = (T*)h->updv;
-  const T* arena = (const T*)h->arena;
   Prof pr(h, prof_cls, s);
   if (A.ilu && h->il_packed) {  // (L~ U~)^-1 y in one launch (the blocks keep their row order)
     launch_ilu_solve<T>(A.p, h->il_max_rows, h->il_max_level, h->il_max_starts, h->il_l, h->il_u,
@@ -771,35 +809,23 @@ void block_solve_impl(ddps_handle* h, const double* y, double* g, cudaStream_t s
     h->launches += 2 + (int64_t)A.il_lf_ptr.size() - 1 + (int64_t)A.il_lb_ptr.size() - 1;
     return;
   }
-  // levels >= top: one persistent launch per sweep; the levels above: one launch each
-  const int top = h->persist_L >= 0 ? h->persist_L : A.nlevels;
-  const int64_t nf = (int64_t)A.f_k.size();
-  int32_t* done_f = h->p_flags;
-  int32_t* done_b = h->p_flags + nf;
-  if (h->persist_L >= 0) {
-    CK(cudaMemsetAsync(h->p_flags, 0, (2 * nf + 2) * sizeof(int32_t), s));
-    launch_fwd_persist<T>(h->F, h->p_fwd, h->persist_n, h->persist_max_m, arena, w, u, done_f,
-                          h->p_flags + 2 * nf, h->derr, s);
-    h->launches++;
-  }
-  for (int L = top - 1; L >= 0; --L)
-    launch_fwd1<T>(h->F, h->level_fronts + A.level_ptr[L], A.level_ptr[L + 1] - A.level_ptr[L],
-                   h->split[L].max_m, arena, w, u, s, h->tune_fwd.empty() ? SOLVE_AUTO : h->tune_fwd[L]);
-  for (int L = 0; L < top; ++L)
-    launch_bwd1<T>(h->F, h->level_fronts + A.level_ptr[L], A.level_ptr[L + 1] - A.level_ptr[L],
-                   h->split[L].max_m, arena, w, s, h->tune_bwd.empty() ? SOLVE_AUTO : h->tune_bwd[L]);
-  if (h->persist_L >= 0) {
-    launch_bwd_persist<T>(h->F, h->p_bwd, h->persist_n, h->persist_max_m, h->p_wait, arena, w,
-                          done_b, h->p_flags + 2 * nf + 1, h->derr, s);
-    h->launches++;
+  // the sweeps on the handle's work vectors are the same launches every time: replayed
+  // from a graph (one launch in place of two per depth, which cost the host more than the
+  // GPU on small problems)
+  if (w == (T*)h->w && u == (T*)h->updv && (h->tuned || h->opt.autotune == 0) && replays_in(h, s)) {
+    if (!h->g_sweeps)
+      h->g_sweeps = capture_graph(h, [&](cudaStream_t gs) { sweep_launches<T>(h, w, u, gs); },
+                                  &h->g_sweeps_launches);
+    replay_graph(h, h->g_sweeps, h->g_sweeps_launches, s);
+  } else {
+    sweep_launches<T>(h, w, u, s);
   }
   launch_permute_out<T>(w, h->perm, A.n, g, s);
-  h->launches += 2 + 2 * top;
+  h->launches += 2;
 }
 
 // ---------------------------------------------------------------------------
-// Autotuner of the block-solve launch shapes.  For every depth above the
-// persistent sweeps and both sweeps, each candidate shape (warp per front
+// Autotuner of the block-solve launch shapes.  For every depth and both sweeps, each candidate shape (warp per front
 // when the fronts allow, one CTA with eight loads in flight, clusters of 1,
 // 2, 4 and 8 CTAs) is timed with CUDA events on the handle's own factors
 // (one untimed launch, then the mean of three), and the fastest is kept.
@@ -849,7 +875,6 @@ void tune_cache_write() {
 template <typename T>
 void autotune_block_solve(ddps_handle* h, cudaStream_t s) {
   const Analysis& A = h->A;
-  const int top = h->persist_L >= 0 ? h->persist_L : A.nlevels;
   h->tune_fwd.assign(A.nlevels, SOLVE_AUTO);
   h->tune_bwd.assign(A.nlevels, SOLVE_AUTO);
   h->tune_fwd_ms.assign(A.nlevels, 0.f);
@@ -867,7 +892,7 @@ void autotune_block_solve(ddps_handle* h, cudaStream_t s) {
   std::lock_guard<std::mutex> lock(g_tune_mutex);
   tune_cache_read();
   bool added = false;
-  for (int L = 0; L < top; ++L) {
+  for (int L = 0; L < A.nlevels; ++L) {
     const int32_t nf = A.level_ptr[L + 1] - A.level_ptr[L];
     const int32_t mm = h->split[L].max_m;
     int64_t ent = 0;
@@ -911,6 +936,34 @@ void autotune_block_solve(ddps_handle* h, cudaStream_t s) {
       }
       (sweep ? h->tune_bwd : h->tune_fwd)[L] = best;
       (sweep ? h->tune_bwd_ms : h->tune_fwd_ms)[L] = best_ms;
+    }
+  }
+  // both sweeps with the deep levels in persistent launches, or every level in its own
+  if (h->persist_L >= 0) {
+    const std::string key = std::string(prop.name) + "|" + std::to_string(sizeof(T)) +
+                            "|persist|" + std::to_string(A.nlevels) + "|" +
+                            std::to_string(h->persist_n) + "|" +
+                            std::to_string(A.factor_lu_entries);
+    auto it = g_tune_cache.find(key);
+    if (it != g_tune_cache.end()) {
+      h->use_persist = it->second == 1;
+    } else {
+      float ms[2];
+      const int64_t l0 = h->launches;
+      for (int v = 0; v < 2; ++v) {
+        h->use_persist = v == 1;
+        sweep_launches<T>(h, w, u, s);
+        CK(cudaEventRecord(e0, s));
+        for (int r = 0; r < 3; ++r) sweep_launches<T>(h, w, u, s);
+        CK(cudaEventRecord(e1, s));
+        CK(cudaEventSynchronize(e1));
+        CK(cudaEventElapsedTime(&ms[v], e0, e1));
+      }
+      h->launches = l0;
+      check_launch();
+      h->use_persist = ms[1] < ms[0];
+      g_tune_cache[key] = h->use_persist ? 1 : 0;
+      added = true;
     }
   }
   // CSR product kernels for A (outer iteration) and R~ (retrieval), timed on
@@ -1239,7 +1292,7 @@ void precond_apply(ddps_handle* h, const double* y, double* z, cudaStream_t s, b
                    bool masked) {
   const int64_t m = (int64_t)h->A.c.size();
   if (h->use_direct && m > 0) {
-    if (graphs_on(h)) {
+    if (replays_in(h, s)) {
       ddps_handle::PrecGraph* pg = nullptr;
       for (auto& q : h->g_prec)
         if (q.y == y && q.z == z) pg = &q;
@@ -2132,6 +2185,9 @@ void build_device(ddps_handle* h, const int32_t* rowptr, const int32_t* colind) 
       h->p_bwd = dupload(h, bwd);
       h->p_wait = dupload(h, wait);
       h->p_flags = dalloc<int32_t>(h, 2 * nf + 2);
+      // without the autotuner: many fronts (70,731 of a 256-system batch take 308 us
+      // against 420 in launches per depth; 514 of a 127 x 127 grid 126 against 72)
+      h->use_persist = h->persist_n >= 16384;
     }
   }
   std::vector<int32_t> gcols_panel(A.gcols.size());
@@ -2611,7 +2667,7 @@ ddps_status ddps_get_tuning(const ddps_handle* h, char* buf, int64_t cap, int64_
   std::ostringstream o;
   static const char* csr[] = {"stream", "vec4", "vec8", "block", "warp"};
   o << "{\"tuned\": " << (h->tuned ? "true" : "false") << ", \"persistent_from_level\": "
-    << h->persist_L << ", \"spmv\": \"" << csr[h->tune_spmv] << "\", \"spmv_ms\": "
+    << (h->use_persist ? h->persist_L : -1) << ", \"spmv\": \"" << csr[h->tune_spmv] << "\", \"spmv_ms\": "
     << h->tune_spmv_ms << ", \"rt_residual\": \"" << csr[h->tune_rt] << "\", \"levels\": [";
   for (size_t L = 0; L < h->tune_fwd.size(); ++L) {
     const int f = h->tune_fwd[L], b = h->tune_bwd[L];
@@ -2701,13 +2757,12 @@ ddps_status ddps_destroy(ddps_handle* h) {
   if (!h) return DDPS_OK;
   if (h->g_inner) cudaGraphExecDestroy(h->g_inner);
   if (h->g_factor) cudaGraphExecDestroy(h->g_factor);
+  if (h->g_sweeps) cudaGraphExecDestroy(h->g_sweeps);
   for (auto& q : h->g_prec) cudaGraphExecDestroy(q.exec);
   if (h->gstream) {
     cudaStreamSynchronize(h->gstream);
     cudaStreamDestroy(h->gstream);
   }
-  for (cudaEvent_t e : h->gev)
-    if (e) cudaEventDestroy(e);
   for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
   for (void* p : h->allocs) cudaFree(p);
   if (h->herr) cudaFreeHost(h->herr);
