@@ -87,7 +87,7 @@ typedef enum { DDPS_REDUCED_ITERATIVE = 0, DDPS_REDUCED_DIRECT = 1 } ddps_reduce
  * ILU0: incomplete LU with zero fill on the pattern of every block, in the
  * block's own row order; G = D~^-1 R~ then uses D~ = L~ U~, and the outer
  * Krylov iteration absorbs the approximation (P = D~ + R~ is no longer A
- * even without dropping).  Spike products run in factor_prec (SIMT). */
+ * even without dropping).  Spike products run in factor_prec. */
 typedef enum { DDPS_FACTOR_LU = 0, DDPS_FACTOR_ILU0 = 1 } ddps_factor_kind;
 
 typedef struct {
@@ -96,8 +96,9 @@ typedef struct {
   int32_t factor_prec;    /* FP64 or FP32: storage and arithmetic of the block factors (Fig. 2 step 2)
                              and of the block solves 6.1 / 6.5 */
   int32_t spike_prec;     /* operands of the spike products of Fig. 2 step 4: equal to factor_prec
-                             (SIMT), or, with FP32 factors, BF16 / BF16X3 (tensor cores, fp32
-                             accumulation) */
+                             (FP64: exact sums of 55-bit fixed-point operands, rounded once;
+                             FP32: SIMT), or, with FP32 factors, BF16 / BF16X3 (tensor cores,
+                             fp32 accumulation) */
   int32_t ghat_prec;      /* FP64, FP32, FP16 or BF16 storage of G^ (Sec. 3: dense per-partition
                              arrays); FP16/BF16 products accumulate in FP32 */
   int32_t inner_prec;     /* FP64 or FP32 vectors of the inner BiCGStab on G^ (6.3) */
