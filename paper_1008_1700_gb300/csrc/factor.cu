@@ -752,7 +752,7 @@ void launch_front_lu_small(DevFronts F, const int32_t* list, int32_t nf, int32_t
                            cudaStream_t s) {
   if (nf <= 0) return;
   const size_t sm = ((size_t)max_m * max_m + 2 * (size_t)max_m) * sizeof(T) + (size_t)max_m * sizeof(double);
-  if (sm > 48 * 1024)
+  if (sm > 40 * 1024)  // static bytes count too
     record_launch_error(cudaFuncSetAttribute(k_front_lu_small<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   k_front_lu_small<T><<<nf, kThreads, sm, s>>>(F, list, arena, rownorm_new, pivot_tol, err);
 }

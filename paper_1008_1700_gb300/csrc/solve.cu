@@ -1058,7 +1058,8 @@ static int sm_count() { return device_sm_count(); }
 // and kSolveB loads per lane.
 template <typename K, typename... Args>
 static void launch_clustered(K kern, int32_t nf, int c, size_t sm, cudaStream_t s, Args... args) {
-  if (sm > 48 * 1024)
+  // the 48 KB that need no opt-in hold the kernel's static shared memory too
+  if (sm > 40 * 1024)
     record_launch_error(
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   cudaLaunchConfig_t cfg = {};
@@ -1253,7 +1254,7 @@ void launch_ghat_matvec_tiled(const TG* ghat, const int32_t* tile_block, const i
   if (ntiles <= 0) return;
   using AT = typename Acc<TG>::type;
   const size_t sm = (size_t)std::max<int64_t>(max_cols, 1) * sizeof(AT);
-  if (sm > 48 * 1024)
+  if (sm > 40 * 1024)  // static bytes count too
     record_launch_error(cudaFuncSetAttribute(k_ghat_matvec_tiled<TG, TI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)sm));
   k_ghat_matvec_tiled<TG, TI><<<ntiles, 256, sm, s>>>(ghat, tile_block, tile_row, tile_h, gq0, gq1,

@@ -162,3 +162,24 @@ def test_reduced_solve_paths(name, N_, p, form):
             q0, q1, cols = S.ghat_layout(b)
             r[q0:q1] -= S.ghat_block(b) @ z[cols]
         assert np.linalg.norm(r) <= 1.1e-5 * np.linalg.norm(g), (name, scale)
+
+
+@pytest.mark.parametrize("autotune", [0, 1])
+@pytest.mark.parametrize("rows", [1004, 1024, 2048])
+def test_block_solve_front_at_48_kb(rows, autotune):
+    """Dense fronts whose sweeps take just under 48 KB of dynamic shared memory (static bytes
+    of the kernel beside it)."""
+    rng = np.random.default_rng(rows)
+    n = rows + 4
+    A = np.zeros((n, n))
+    A[:rows, :rows] = rng.uniform(-1.0, 1.0, (rows, rows))
+    A[0, rows] = A[rows, 0] = 1.0
+    A[np.arange(n), np.arange(n)] = 2.0 * rows
+    M = sp.csr_matrix(A)
+    S = Solver(M.indptr, M.indices, np.array([0, rows, n]), factor_prec=N.DDPS_FP64,
+               spike_prec=N.DDPS_FP64, ghat_prec=N.DDPS_FP64, inner_prec=N.DDPS_FP64,
+               autotune=autotune)
+    S.factor(dev(M.data))
+    x, _ = S.solve(dev(A @ np.ones(n)))
+    # dominance 2: condition below 3, |x - 1| <= 3 (n + rounding of the right-hand side) eps
+    assert np.max(np.abs(host(x) - 1.0)) <= 3 * 2 * n * 2.0 ** -53 + 1e-12
