@@ -40,6 +40,7 @@ namespace {
 constexpr int OZ_D = 7, OZ_L = 8;           // digits, levels
 constexpr int OZ_R = oz_tile_m(), OZ_C = 128, OZ_T = 512;  // front rows (N) and panel columns (M) of a tile
 constexpr int OZ_RPT = OZ_R * OZ_C / OZ_T, OZ_KPT = TC_BK * OZ_C / OZ_T;  // rows of C, of a stage of B per thread
+static_assert(OZ_R % TC_BK == 0, "a tile's first row starts a stage of K");
 static_assert(OZ_RPT == 8 && OZ_KPT % 4 == 0, "shares of a thread");
 constexpr int OZ_GROUP = 4;                 // stages of 32 between two drains: 128 values of K
 constexpr uint32_t OZ_ATILE = OZ_R * TC_BK * 2, OZ_BTILE = OZ_C * TC_BK * 2;
@@ -265,8 +266,10 @@ __global__ void __launch_bounds__(OZ_T, 2)
   const int M = OP == OP_FWD_L21 ? m - k : k, K = OP == OP_BWD_U12 ? m - k : k;
   const int rows = min(OZ_R, M - m0);
   const int32_t* __restrict__ idx = F.idx + tb0;
-  int nk = (K + TC_BK - 1) / TC_BK;
-  const unsigned char* apk = head + OZ_HEAD;
+  // the triangles' columns of these rows: up to the last row's (L11^-1), from the first (U11^-1)
+  const int k0 = OP == OP_BWD_UINV ? m0 : 0, k1 = OP == OP_FWD_LINV ? min(K, m0 + OZ_R) : K;
+  int nk = (k1 - k0 + TC_BK - 1) / TC_BK;
+  const unsigned char* apk = head + OZ_HEAD + (int64_t)(k0 / TC_BK) * OZ_ABLK;
   const uint32_t sbase = smem_u32(smem);
   int issued = 0, committed = 0;  // thread 0
   auto fetch_a = [&](int kt) {
@@ -296,10 +299,10 @@ __global__ void __launch_bounds__(OZ_T, 2)
   double breg[OZ_KPT];
   int ureg[OZ_KPT];
   auto load_b = [&](int kt) {
-    const int g0 = kt * TC_BK + bk * OZ_KPT;
+    const int g0 = k0 + kt * TC_BK + bk * OZ_KPT;
 #pragma unroll
     for (int t = 0; t < OZ_KPT; ++t) {
-      const bool in = g0 + t < K;
+      const bool in = g0 + t < k1;
       breg[t] = live && in ? Bp[brow(g0 + t) * NR + n0 + bc] : 0.0;
       ureg[t] = in ? oz_unit<OP>(U, idx, row0, k, g0 + t) : 0;
     }

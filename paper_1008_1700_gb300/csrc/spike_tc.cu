@@ -161,7 +161,10 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
   const int64_t row0 = F.row0[f];
   const int64_t tb0 = F.idx_off[f];
   const int32_t* __restrict__ idx = F.idx + F.idx_off[f];
-  const unsigned char* apk = atc + tile_aoff[blockIdx.x];
+  // the triangles' columns of these rows: up to the last row's (L11^-1), from the first
+  // (U11^-1); the zeros beyond them took half of these products' time
+  const int kb = OP == OP_BWD_UINV ? m0 : 0, ke = OP == OP_FWD_LINV ? min(d.K, m0 + TC_BM) : d.K;
+  const unsigned char* apk = atc + tile_aoff[blockIdx.x] + (int64_t)(kb / TC_BK) * kAB;
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -184,14 +187,14 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
   const uint32_t sbase = smem_u32(smem);
   bool timed_out = false;
 
-  int nk = (d.K + TC_BK - 1) / TC_BK;
+  int nk = (ke - kb + TC_BK - 1) / TC_BK;
   // B (panel rows, fp32) of one stage: each thread holds kBItems runs of 8
   // K-consecutive values of one column in registers, loaded one stage ahead
   constexpr int kBItems = (TC_BN * TC_BK / 8) / TC_THREADS;
   float breg[kBItems][8];
   const float* Bp = (OP == OP_FWD_L21 || OP == OP_BWD_U12) ? X : Tb;
   auto load_b = [&](int kt) {
-    const int k0 = kt * TC_BK;
+    const int k0 = kb + kt * TC_BK;
 #pragma unroll
     for (int q = 0; q < kBItems; ++q) {
       const int e = tid + q * TC_THREADS;
@@ -201,7 +204,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
       for (int t = 0; t < 8; ++t) {
         const int gk = k0 + kc * 8 + t;
         float val = 0.f;
-        if (gk < d.K && gj < ncols) {
+        if (gk < ke && gj < ncols) {
           int64_t brow;
           if (OP == OP_FWD_LINV || OP == OP_BWD_UINV)
             brow = tb0 + gk;
