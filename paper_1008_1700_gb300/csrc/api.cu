@@ -57,6 +57,11 @@ size_t prec_size(int prec) { return prec == DDPS_FP64 ? 8 : (prec == DDPS_FP32 ?
 
 // Fronts of one depth reordered for the LU launches: `nsmall` fronts that fit
 // the shared-memory kernel, then `nlarge` others, starting at `first`.
+// FP32 fronts of more pivots get their triangular inverses by doubling on the tensor cores
+// (build_inverse_products); at up to 512 either way takes the same time within 1% of the
+// block LU (64^3, 48^3, 300k band).
+constexpr int32_t kInvTcK = 256;
+
 struct LevelSplit {
   int32_t first = 0, nsmall = 0, nlarge = 0, max_small_m = 0, max_m = 0;
   // multi-CTA LU of the large fronts: per panel step p (columns 32p..32p+31),
@@ -70,6 +75,11 @@ struct LevelSplit {
   // lu_pc_front / lu_pc_word
   std::vector<int64_t> pq_ptr;
   int32_t inv_first = 0, inv_ntiles = 0;  // multi-CTA inverse tiles of the large fronts
+  // doubling steps of the wide fronts' inverses on the tensor cores: launch q takes the
+  // problems [gm_ptr[q], gm_ptr[q + 1]) of inv_gemm and gm_tiles[q] tiles
+  std::vector<int64_t> gm_ptr;
+  int64_t gm_first = 0;  // launches of the depths before (their prefixes have an entry more)
+  std::vector<int32_t> gm_tiles;
 };
 
 struct ddps_handle {
@@ -138,7 +148,9 @@ struct ddps_handle {
   void* lu_dinv = nullptr;  // 32 x 32 inverses of the panel's diagonal triangles, per front
   bool lu_tc = false;
   int32_t *inv_tile_front = nullptr, *inv_tile_cb = nullptr;
-  int64_t* inv_off = nullptr;  // per front, offset of its 2 k^2 inverse entries in inv
+  int64_t* inv_off = nullptr;  // per front, offset of its two inverses in inv
+  GemmDesc* inv_gemm = nullptr;
+  int32_t* inv_prefix = nullptr;  // per launch, first tile of each of its problems, then the total
   void* inv = nullptr;
   // spike GEMM tile lists per depth: backward tiles over the k pivot rows (tk),
   // forward tiles over the pivot rows (fk) and over the r update rows (tr).
@@ -642,9 +654,16 @@ void factor_launches(ddps_handle* h, cudaStream_t s) {
         }
       }
       launch_tri_inverse_mc<T>(h->F, h->inv_tile_front + ls.inv_first, h->inv_tile_cb + ls.inv_first,
-                               ls.inv_ntiles, h->lu_order + ls.first + ls.nsmall, ls.nlarge, h->max_k,
-                               arena, (T*)h->inv, h->inv_off, s);
-      h->launches += 2;
+                               ls.inv_ntiles, ls.gm_tiles.empty() ? INT32_MAX : kInvTcK, arena,
+                               (T*)h->inv, h->inv_off, s);
+      for (size_t q = 0; q < ls.gm_tiles.size(); ++q) {
+        launch_gemm_grouped_tc(h->inv_gemm + ls.gm_ptr[q], h->inv_prefix + ls.gm_ptr[q] + ls.gm_first + q,
+                               (int32_t)(ls.gm_ptr[q + 1] - ls.gm_ptr[q]), ls.gm_tiles[q], h->derr, s);
+        h->launches++;
+      }
+      launch_tri_inverse_copy<T>(h->F, h->lu_order + ls.first + ls.nsmall, ls.nlarge, h->max_k, arena,
+                                 (const T*)h->inv, h->inv_off, s);
+      h->launches += 3;
     }
   }
   launch_gather_rt_values(h->vals, h->rt_src, h->nrt, h->rt_val, s);
@@ -1794,6 +1813,62 @@ bool oz_wins(const Analysis& A) {
   return bytes <= (int64_t)24 << 30;
 }
 
+// Triangular inverses of the wide FP32 fronts from those of their diagonal blocks, two
+// neighbours at a time: X21 = -X22 (L21 X11) and X12 = -X11 (U12 X22), b = 128, 256, ..
+// pivots each, as one launch of products per step and factor over all fronts of a depth.  The
+// inner products go to the same place of the other inverse, whose half is free.  (The GEMMs
+// are row-major: they form the transposes of these column-major blocks.)
+void build_inverse_products(ddps_handle* h, const std::vector<int32_t>& order,
+                            const std::vector<int64_t>& ioff) {
+  const Analysis& A = h->A;
+  float* arena = (float*)h->arena;
+  std::vector<GemmDesc> desc;
+  std::vector<int32_t> prefix;
+  int64_t launches = 0;
+  for (LevelSplit& ls : h->split) {
+    ls.gm_first = launches;
+    ls.gm_ptr.assign(1, (int64_t)desc.size());
+    int32_t kmax = 0;
+    for (int32_t t = 0; t < ls.nlarge; ++t) kmax = std::max(kmax, A.f_k[order[ls.first + ls.nsmall + t]]);
+    if (kmax <= kInvTcK) continue;
+    for (int64_t b = kInvGroup; b < kmax; b *= 2)
+      for (int step = 0; step < 2; ++step) {
+        int32_t tiles = 0;
+        auto add = [&](const float* a, int64_t lda, const float* bb, int64_t ldb, float* c, int64_t ldc,
+                       int64_t M, int64_t N, int64_t K, float alpha, int32_t tri) {
+          prefix.push_back(tiles);
+          desc.push_back(GemmDesc{a, bb, c, (int32_t)M, (int32_t)N, (int32_t)K, (int32_t)lda, (int32_t)ldb,
+                                  (int32_t)ldc, alpha, 0.f, tri});
+          tiles += (int32_t)(((M + 127) / 128) * ((N + 127) / 128));
+        };
+        for (int32_t t = 0; t < ls.nlarge; ++t) {
+          const int32_t f = order[ls.first + ls.nsmall + t];
+          const int64_t k = A.f_k[f], m = A.f_m[f], ld = inv_ld((int32_t)k);
+          if (k <= kInvTcK) continue;
+          const float* G = arena + A.f_arena[f];
+          float *Lo = (float*)h->inv + ioff[f], *Up = Lo + ld * k;
+          for (int64_t i = 0; i + b < k; i += 2 * b) {
+            const int64_t i2 = i + b, n2 = std::min(b, k - i2);
+            float *T21 = Up + i2 + i * ld, *T12 = Lo + i + i2 * ld;
+            if (step == 0) {
+              add(Lo + i + i * ld, ld, G + i2 + i * m, m, T21, ld, b, n2, b, 1.f, GEMM_FROM_M);
+              add(Up + i2 + i2 * ld, ld, G + i + i2 * m, m, T12, ld, n2, b, n2, 1.f, GEMM_TO_M);
+            } else {
+              add(T21, ld, Lo + i2 + i2 * ld, ld, Lo + i2 + i * ld, ld, b, n2, n2, -1.f, GEMM_TO_N);
+              add(T12, ld, Up + i + i * ld, ld, Up + i + i2 * ld, ld, n2, b, b, -1.f, GEMM_FROM_N);
+            }
+          }
+        }
+        prefix.push_back(tiles);
+        ls.gm_ptr.push_back((int64_t)desc.size());
+        ls.gm_tiles.push_back(tiles);
+        ++launches;
+      }
+  }
+  h->inv_gemm = dupload(h, desc);
+  h->inv_prefix = dupload(h, prefix);
+}
+
 void build_device(ddps_handle* h, const int32_t* rowptr, const int32_t* colind) {
   Analysis& A = h->A;
   const int64_t n = A.n, m = (int64_t)A.c.size();
@@ -1961,7 +2036,7 @@ void build_device(ddps_handle* h, const int32_t* rowptr, const int32_t* colind) 
       for (int32_t i = ls.first + ls.nsmall; i < (int32_t)order.size(); ++i) {
         const int32_t f = order[i];
         ioff[f] = inv_total;
-        inv_total += 2 * (int64_t)A.f_k[f] * A.f_k[f];
+        inv_total += 2 * (int64_t)inv_ld(A.f_k[f]) * A.f_k[f];
         for (int32_t cb = 0; cb * kInvBlock < A.f_k[f]; ++cb) {
           ivf.push_back(f);
           ivc.push_back(cb);
@@ -2021,7 +2096,12 @@ void build_device(ddps_handle* h, const int32_t* rowptr, const int32_t* colind) 
     h->inv_tile_front = dupload(h, ivf);
     h->inv_tile_cb = dupload(h, ivc);
     h->inv_off = dupload(h, ioff);
-    h->inv = dalloc_bytes(h, std::max<int64_t>(inv_total, 1) * (int64_t)prec_size(h->opt.factor_prec));
+    {
+      const int64_t bytes = std::max<int64_t>(inv_total, 1) * (int64_t)prec_size(h->opt.factor_prec);
+      h->inv = dalloc_bytes(h, bytes);
+      CK(cudaMemset(h->inv, 0, bytes));  // the diagonal blocks' other triangles stay zero
+    }
+    if (h->opt.factor_prec == DDPS_FP32) build_inverse_products(h, order, ioff);
     h->lu_panel_fronts = dupload(h, pfronts);
     h->lu_tile_front = dupload(h, tfront);
     h->lu_tile_ij = dupload(h, tij);

@@ -299,14 +299,17 @@ __global__ void __launch_bounds__(kThreads)
 
 // ---------------------------------------------------------------------------
 // Triangular inverses of large fronts with many CTAs, out of place into
-// `inv` (k x k column-major per front at inv_off[f]; L11^-1, then U11^-1).
+// `inv` (two inv_ld(k) x k column-major blocks per front at inv_off[f]: L11^-1, then U11^-1).
 // The diagonal 64 x 64 tiles of an inverse are the inverses of the diagonal
 // tiles of the triangle: k_tri_inverse_diag forms them first, one CTA per
 // tile.  Then CTA (front, column block of 64) of k_tri_inverse_mc walks its
 // column block away from the diagonal: tile X(i, j) = -D(i)^-1 sum_l A(i, l)
 // X(l, j) over the tiles l already solved, as two tile GEMMs (D(i)^-1 is the
-// diagonal tile of X).  k_tri_inverse_copy then writes the strictly lower
-// part of L11^-1 and the upper part of U11^-1 back into the front.
+// diagonal tile of X).  The walk is a chain of k / 64 steps on the FP32 cores (17 TFLOP/s);
+// for FP32 fronts of more than wide_k pivots it stops at the diagonal 128 x 128 blocks, and
+// the grouped tensor-core products double these (as exact as FP32 FMAs).  300k band, fronts
+// of up to 4,227 pivots: 57.4 -> 11.1 ms of a factorisation.  k_tri_inverse_copy then writes
+// the strictly lower part of L11^-1 and the upper part of U11^-1 back into the front.
 // ---------------------------------------------------------------------------
 constexpr int IB = 64;  // columns per CTA and rows per tile
 
@@ -320,7 +323,8 @@ __global__ void __launch_bounds__(kThreads)
   const int i0 = tile_cb[blockIdx.x] * IB;
   const bool upper = blockIdx.y == 1;
   const T* __restrict__ A = arena + F.arena[f];
-  T* __restrict__ X = inv + inv_off[f] + (upper ? (int64_t)k * k : 0);
+  const int32_t ld = inv_ld(k);
+  T* __restrict__ X = inv + inv_off[f] + (upper ? (int64_t)ld * k : 0);
   const int tid = threadIdx.x;
   // two 64 x 65 tiles of dynamic shared memory (the triangle's tile, the inverse)
   extern __shared__ unsigned char smem_raw[];
@@ -355,21 +359,23 @@ __global__ void __launch_bounds__(kThreads)
   }
   for (int t = tid; t < IB * IB; t += blockDim.x) {
     const int r = t % IB, c = t / IB;
-    if (r < rows && c < rows) X[(i0 + r) + (int64_t)(i0 + c) * k] = Ts[r][c];
+    if (r < rows && c < rows) X[(i0 + r) + (int64_t)(i0 + c) * ld] = Ts[r][c];
   }
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
     k_tri_inverse_mc(DevFronts F, const int32_t* __restrict__ tile_front,
-                     const int32_t* __restrict__ tile_cb, const T* __restrict__ arena,
-                     T* __restrict__ inv, const int64_t* __restrict__ inv_off) {
+                     const int32_t* __restrict__ tile_cb, int32_t wide_k,
+                     const T* __restrict__ arena, T* __restrict__ inv,
+                     const int64_t* __restrict__ inv_off) {
   const int32_t f = tile_front[blockIdx.x];
   const int32_t k = F.k[f], m = F.m[f];
   const int j0 = tile_cb[blockIdx.x] * IB;
   const bool upper = blockIdx.y == 1;
   const T* __restrict__ A = arena + F.arena[f];
-  T* __restrict__ X = inv + inv_off[f] + (upper ? (int64_t)k * k : 0);
+  const int32_t ld = inv_ld(k);
+  T* __restrict__ X = inv + inv_off[f] + (upper ? (int64_t)ld * k : 0);
   const int tid = threadIdx.x;
   extern __shared__ unsigned char smem_raw[];
   T(*As)[NB + 1] = reinterpret_cast<T(*)[NB + 1]>(smem_raw);
@@ -379,7 +385,12 @@ __global__ void __launch_bounds__(kThreads)
   T(*Ds)[IB + 1] = reinterpret_cast<T(*)[IB + 1]>(
       smem_raw + sizeof(T) * (IB * (NB + 1) + NB * (IB + 1) + IB * (IB + 1)));
   const int tr = tid % 16, tc = tid / 16;
-  const int ntile_rows = upper ? (min(j0 + IB, k) + IB - 1) / IB : (k - j0 + IB - 1) / IB;
+  int ntile_rows = upper ? (min(j0 + IB, k) + IB - 1) / IB : (k - j0 + IB - 1) / IB;
+  if (k > wide_k) {  // within the diagonal block of kInvGroup only
+    const int q = j0 % kInvGroup / IB;
+    ntile_rows = min(ntile_rows, upper ? q + 1 : kInvGroup / IB - q);
+  }
+  if (ntile_rows <= 1) return;
   // it = 0 is the diagonal tile, formed by k_tri_inverse_diag
   for (int it = 1; it < ntile_rows; ++it) {
     // lower: row tiles below j0 downwards; upper: above the diagonal tile upwards
@@ -399,7 +410,7 @@ __global__ void __launch_bounds__(kThreads)
         As[r][q] = (gi < k && gl < l_end) ? A[gi + (int64_t)gl * m] : T(0);
         const int q2 = t % NB, c2 = t / NB;
         const int gl2 = l0 + q2, gj = j0 + c2;
-        Bs[q2][c2] = (gl2 < l_end && gj < k) ? X[gl2 + (int64_t)gj * k] : T(0);
+        Bs[q2][c2] = (gl2 < l_end && gj < k) ? X[gl2 + (int64_t)gj * ld] : T(0);
       }
       __syncthreads();
 #pragma unroll 8
@@ -424,7 +435,7 @@ __global__ void __launch_bounds__(kThreads)
       for (int b2 = 0; b2 < 4; ++b2) Ts[tr + 16 * a2][tc + 16 * b2] = -acc[a2][b2];
     for (int t = tid; t < IB * IB; t += blockDim.x) {
       const int r = t % IB, c = t / IB;
-      Ds[r][c] = (r < rows && c < rows) ? X[(i0 + r) + (int64_t)(i0 + c) * k] : T(0);
+      Ds[r][c] = (r < rows && c < rows) ? X[(i0 + r) + (int64_t)(i0 + c) * ld] : T(0);
     }
     __syncthreads();
 #pragma unroll
@@ -448,7 +459,7 @@ __global__ void __launch_bounds__(kThreads)
 #pragma unroll
       for (int b2 = 0; b2 < 4; ++b2) {
         const int r = tr + 16 * a2, c = tc + 16 * b2;
-        if (r < rows && j0 + c < k) X[(i0 + r) + (int64_t)(j0 + c) * k] = acc[a2][b2];
+        if (r < rows && j0 + c < k) X[(i0 + r) + (int64_t)(j0 + c) * ld] = acc[a2][b2];
       }
     __syncthreads();
   }
@@ -461,12 +472,14 @@ __global__ void k_tri_inverse_copy(DevFronts F, const int32_t* __restrict__ list
   const int32_t f = list[blockIdx.y];
   const int32_t k = F.k[f], m = F.m[f];
   T* __restrict__ A = arena + F.arena[f];
+  const int32_t ld = inv_ld(k);
   const T* __restrict__ X = inv + inv_off[f];
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < (int64_t)k * k;
        t += (int64_t)gridDim.x * blockDim.x) {
     const int i = (int)(t % k), j = (int)(t / k);
-    // lower inverse sits in the first k*k entries, upper inverse in the next k*k
-    A[i + (int64_t)j * m] = i > j ? X[t] : X[(int64_t)k * k + t];
+    // lower inverse first, then the upper one
+    const int64_t e = i + (int64_t)j * ld;
+    A[i + (int64_t)j * m] = i > j ? X[e] : X[(int64_t)ld * k + e];
   }
 }
 
@@ -730,8 +743,8 @@ void launch_lu_trailing(DevFronts F, const int32_t* tile_front, const int32_t* t
 
 template <typename T>
 void launch_tri_inverse_mc(DevFronts F, const int32_t* tile_front, const int32_t* tile_cb,
-                           int32_t ntiles, const int32_t* list, int32_t nf, int32_t max_k, T* arena,
-                           T* inv, const int64_t* inv_off, cudaStream_t s) {
+                           int32_t ntiles, int32_t wide_k, const T* arena, T* inv,
+                           const int64_t* inv_off, cudaStream_t s) {
   if (ntiles <= 0) return;
   const size_t sm = sizeof(T) * ((size_t)IB * (NB + 1) + (size_t)NB * (IB + 1) + 2 * (size_t)IB * (IB + 1));
   record_launch_error(cudaFuncSetAttribute(k_tri_inverse_mc<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
@@ -739,8 +752,14 @@ void launch_tri_inverse_mc(DevFronts F, const int32_t* tile_front, const int32_t
   record_launch_error(cudaFuncSetAttribute(k_tri_inverse_diag<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smd));
   k_tri_inverse_diag<T><<<dim3(ntiles, 2), kThreads, smd, s>>>(F, tile_front, tile_cb, arena, inv,
                                                                 inv_off);
-  k_tri_inverse_mc<T><<<dim3(ntiles, 2), kThreads, sm, s>>>(F, tile_front, tile_cb, arena, inv,
-                                                             inv_off);
+  k_tri_inverse_mc<T><<<dim3(ntiles, 2), kThreads, sm, s>>>(F, tile_front, tile_cb, wide_k, arena,
+                                                             inv, inv_off);
+}
+
+template <typename T>
+void launch_tri_inverse_copy(DevFronts F, const int32_t* list, int32_t nf, int32_t max_k, T* arena,
+                             const T* inv, const int64_t* inv_off, cudaStream_t s) {
+  if (nf <= 0) return;
   const int64_t per = (int64_t)max_k * max_k;
   const int gx = (int)std::min<int64_t>(std::max<int64_t>((per + kThreads - 1) / kThreads, 1), 256);
   k_tri_inverse_copy<T><<<dim3(gx, nf), kThreads, 0, s>>>(F, list, arena, inv, inv_off);
@@ -776,8 +795,9 @@ void launch_ghat_extract(const int32_t* qblock, const int32_t* c_rownew, const i
   template void launch_front_lu_small<T>(DevFronts, const int32_t*, int32_t, int32_t, T*,      \
                                          const double*, double, long long*, cudaStream_t);      \
   template void launch_tri_inverse_mc<T>(DevFronts, const int32_t*, const int32_t*, int32_t,    \
-                                         const int32_t*, int32_t, int32_t, T*, T*,              \
-                                         const int64_t*, cudaStream_t);                         \
+                                         int32_t, const T*, T*, const int64_t*, cudaStream_t);  \
+  template void launch_tri_inverse_copy<T>(DevFronts, const int32_t*, int32_t, int32_t, T*,     \
+                                           const T*, const int64_t*, cudaStream_t);             \
   template void launch_lu_panel<T>(DevFronts, const int32_t*, int32_t, const int32_t*,          \
                                    const int32_t*, const int32_t*, int32_t, int32_t, T*, T*,    \
                                    const double*, double, long long*, cudaStream_t);            \

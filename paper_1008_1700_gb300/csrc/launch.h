@@ -150,12 +150,18 @@ void launch_front_lu_small(DevFronts F, const int32_t* list, int32_t nf, int32_t
 constexpr int kLuPanel = 32;
 constexpr int kLuTile = 64;
 // Multi-CTA triangular inverses of large fronts: tile_front / tile_cb list
-// (front, 64-column block); inv holds 2 k^2 entries per front at inv_off.
-constexpr int kInvBlock = 64;
+// (front, 64-column block); inv holds two inv_ld(k) x k blocks per front at inv_off (a
+// multiple of four).  Fronts of more than wide_k pivots get the inverses of their diagonal
+// 128 x 128 blocks only; launch_tri_inverse_copy then writes them back.
+constexpr int kInvBlock = 64, kInvGroup = 128;
+__host__ __device__ constexpr int32_t inv_ld(int32_t k) { return (k + 3) / 4 * 4; }
 template <typename T>
 void launch_tri_inverse_mc(DevFronts F, const int32_t* tile_front, const int32_t* tile_cb,
-                           int32_t ntiles, const int32_t* list, int32_t nf, int32_t max_k, T* arena,
-                           T* inv, const int64_t* inv_off, cudaStream_t s);
+                           int32_t ntiles, int32_t wide_k, const T* arena, T* inv,
+                           const int64_t* inv_off, cudaStream_t s);
+template <typename T>
+void launch_tri_inverse_copy(DevFronts F, const int32_t* list, int32_t nf, int32_t max_k, T* arena,
+                             const T* inv, const int64_t* inv_off, cudaStream_t s);
 // Panel step j0 of the large fronts in `list`: the diagonal block and the
 // inverses of its triangles (one CTA per front; dinv holds 2 x 32 x 32
 // entries per list entry), then L21 rows and U12 columns over chunks of 256

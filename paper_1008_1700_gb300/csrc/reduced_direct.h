@@ -20,7 +20,11 @@ struct GemmDesc {
   float* C;
   int32_t M, N, K, lda, ldb, ldc;
   float alpha, beta;
+  // zero part of a triangular operand: a 128 x 128 tile at (m0, n0) takes the values of K from
+  // m0 (GEMM_FROM_M), up to m0 + 127 (GEMM_TO_M), from n0 or up to n0 + 127
+  int32_t tri = 0;
 };
+enum { GEMM_FROM_M = 1, GEMM_TO_M = 2, GEMM_FROM_N = 3, GEMM_TO_N = 4 };
 // y = y0 + alpha A x (y0 null: 0)
 struct GemvDesc {
   const float* A;

@@ -540,10 +540,13 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
     const int mid = (lo + hi) >> 1;
     if (prefix[mid] <= (int)blockIdx.x) lo = mid; else hi = mid;
   }
-  const GemmDesc d = D[lo];
+  GemmDesc d = D[lo];
   const int t = blockIdx.x - prefix[lo];
   const int tiles_n = (d.N + TC_BN - 1) / TC_BN;
   const int m0 = (t / tiles_n) * TC_BM, n0 = (t % tiles_n) * TC_BN;
+  if (d.tri == GEMM_TO_M || d.tri == GEMM_TO_N)
+    d.K = min(d.K, (d.tri == GEMM_TO_M ? m0 : n0) + TC_BM);
+  const int kfirst = d.tri == GEMM_FROM_M ? m0 : d.tri == GEMM_FROM_N ? n0 : 0;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -567,7 +570,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
   const bool vec = d.lda % 4 == 0 && ((uintptr_t)d.A & 15) == 0;
   float areg[2][8], breg[2][8];
   auto load = [&](int kt) {
-    const int k0 = kt * TC_BK;
+    const int k0 = kfirst + kt * TC_BK;
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       const int e = tid + q * TC_THREADS;
@@ -620,7 +623,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   };
 
-  const int nk = (d.K + TC_BK - 1) / TC_BK;
+  const int nk = (d.K - kfirst + TC_BK - 1) / TC_BK;
   if (nk > 0) load(0);
   for (int kt = 0; kt < nk; ++kt) {
     const int st = kt & 1;

@@ -183,3 +183,27 @@ def test_block_solve_front_at_48_kb(rows, autotune):
     x, _ = S.solve(dev(A @ np.ones(n)))
     # dominance 2: condition below 3, |x - 1| <= 3 (n + rounding of the right-hand side) eps
     assert np.max(np.abs(host(x) - 1.0)) <= 3 * 2 * n * 2.0 ** -53 + 1e-12
+
+
+@pytest.mark.parametrize("rows", [256, 257, 384, 515, 641, 1301])
+def test_fp32_wide_front_inverses(rows):
+    """Block solves through one dense FP32 front: its triangular inverses come from doubling
+    steps of 128, 256, .. pivots with ragged last blocks and any row stride."""
+    rng = np.random.default_rng(rows)
+    n = rows + 3
+    A = np.zeros((n, n))
+    A[:rows, :rows] = rng.uniform(-1.0, 1.0, (rows, rows))
+    A[0, rows] = A[rows, 0] = 1.0
+    A[np.arange(n), np.arange(n)] = 0.0
+    A[np.arange(n), np.arange(n)] = 1.5 * np.abs(A).sum(axis=1) + 0.1
+    M = sp.csr_matrix(A)
+    S = Solver(M.indptr, M.indices, np.array([0, rows, n]), factor_prec=N.DDPS_FP32,
+               spike_prec=N.DDPS_FP32, ghat_prec=N.DDPS_FP32, inner_prec=N.DDPS_FP32)
+    S.factor(dev(M.data))
+    y = rng.uniform(-1.0, 1.0, n)
+    x = host(S.block_solve(dev(y)))[:rows]
+    r = A[:rows, :rows] @ x - y[:rows]
+    # dominance: |L||U| <= 3 |M|; rows roundings each for the factors, the inverses and the
+    # two triangular products of the solve
+    assert np.linalg.norm(r) <= 3 * 4 * rows * 2.0 ** -24 * np.linalg.norm(np.abs(A[:rows, :rows]) @ np.abs(x))
+    S.close()
