@@ -224,9 +224,11 @@ ddps_status ddps_factor_host(ddps_handle* h, const double* values_host, void* st
  *   f     device float64[n * nrhs]: nrhs right-hand sides, each n contiguous
  *         entries (column-major n x nrhs)
  *   x     device float64[n * nrhs] (output), same layout
- *   nrhs  number of right-hand sides (>= 1); they are solved one after the
- *         other with the same factors (the factor phase needs no right-hand
- *         side, Sec. 3)
+ *   nrhs  number of right-hand sides (>= 1), solved with the same factors (the
+ *         factor phase needs no right-hand side, Sec. 3): one after the other,
+ *         or up to four together (stored G^ of at most 32 bits, iterative reduced
+ *         solve of a system too large for one cluster, no reduced guess set; the
+ *         first such solve allocates their vectors, 4 GB at most)
  *   x0    device float64[n * nrhs] initial guesses, or NULL for x0 = 0; a
  *         guess that already meets tol_out is returned after no iteration
  *   info  host, may be NULL: iterations are the largest over the right-hand

@@ -82,7 +82,38 @@ struct LevelSplit {
   std::vector<int32_t> gm_tiles;
 };
 
-struct ddps_handle {
+// The vectors, scalars and graphs of a solve: of one right-hand side, or of `width` of them
+// that are iterated together (each vector then holds `width` vectors one after the other, and
+// every system of every right-hand side is a segment with scalars of its own).
+constexpr int kMaxWide = 4;
+struct SolveWork {
+  int width = 1;
+  void *w = nullptr, *updv = nullptr;  // block solve: permuted vector, the fronts' update vectors
+  SegView Sn{}, Sm{};
+  int32_t nseg = 0;
+  // outer workspace (FP64, n)
+  double *o_r = nullptr, *o_rhat = nullptr, *o_p = nullptr, *o_v = nullptr, *o_phat = nullptr,
+         *o_s = nullptr, *o_shat = nullptr, *o_t = nullptr, *o_xt = nullptr, *o_tmp = nullptr;
+  // preconditioner workspace
+  double *pc_g = nullptr, *pc_ghat = nullptr, *pc_zhat = nullptr, *pc_t = nullptr;
+  // inner workspace (inner precision, m)
+  void *i_g = nullptr, *i_z = nullptr, *i_r = nullptr, *i_rh = nullptr, *i_p = nullptr,
+       *i_v = nullptr, *i_s = nullptr, *i_t = nullptr;
+  KScal *sc_out = nullptr, *sc_in = nullptr;
+  KScal* hsc = nullptr;      // pinned host scalars of the loop being run (nseg)
+  // Uploads copy hsc into a slot of this pinned ring first, so that the host
+  // may change hsc right after enqueueing an upload; the ring restarts after
+  // every synchronising download.
+  KScal* hstage = nullptr;
+  int stage_next = 0;
+  KScal* hsc_out = nullptr;  // pinned, outer loop
+  KScal* hsc_in = nullptr;   // pinned, inner loop
+  double* partial = nullptr;
+  cudaGraphExec_t g_inner = nullptr, g_sweeps = nullptr;
+  int64_t g_inner_launches = 0, g_sweeps_launches = 0;
+};
+
+struct ddps_handle : SolveWork {
   std::string err;
   ddps_options opt{};
   Analysis A;
@@ -102,8 +133,6 @@ struct ddps_handle {
   int32_t* ea_list = nullptr;
   std::vector<int32_t> ea_maxr;
   void* arena = nullptr;
-  void* updv = nullptr;
-  void* w = nullptr;
   double* rownorm = nullptr;
   long long* derr = nullptr;
   long long* herr = nullptr;  // pinned
@@ -208,30 +237,15 @@ struct ddps_handle {
   bool oz = false;  // FP64 spikes: fixed-point products, digits of A packed in atc
   OzUnits oz_u{};
   int32_t* oz_work = nullptr;
-  // segments
-  SegView Sn{}, Sm{};
-  int32_t nseg = 0;
-  // outer workspace (FP64, n)
-  double *o_r = nullptr, *o_rhat = nullptr, *o_p = nullptr, *o_v = nullptr, *o_phat = nullptr,
-         *o_s = nullptr, *o_shat = nullptr, *o_t = nullptr, *o_xt = nullptr, *o_tmp = nullptr;
-  // preconditioner workspace
-  double *pc_g = nullptr, *pc_ghat = nullptr, *pc_zhat = nullptr, *pc_t = nullptr;
   double *im_q = nullptr, *im_g = nullptr;  // implicit G^: R~ v and D~^-1 R~ v
   // host-buffer entry points stage f and x here
   double *io_f = nullptr, *io_x = nullptr;
-  // inner workspace (inner precision, m)
-  void *i_g = nullptr, *i_z = nullptr, *i_r = nullptr, *i_rh = nullptr, *i_p = nullptr,
-       *i_v = nullptr, *i_s = nullptr, *i_t = nullptr;
-  KScal *sc_out = nullptr, *sc_in = nullptr;
-  KScal* hsc = nullptr;      // pinned host scalars of the loop being run (nseg)
-  // Uploads copy hsc into a slot of this pinned ring first, so that the host
-  // may change hsc right after enqueueing an upload; the ring restarts after
-  // every synchronising download.
-  KScal* hstage = nullptr;
-  int stage_next = 0;
-  KScal* hsc_out = nullptr;  // pinned, outer loop
-  KScal* hsc_in = nullptr;   // pinned, inner loop
-  double* partial = nullptr;
+  // several right-hand sides together (kMaxWide at most; allocated by the first such solve)
+  SolveWork wide;
+  bool wide_ok = false, wide_failed = false;
+  cudaGraphExec_t wide_inner[kMaxWide + 1] = {}, wide_sweeps[kMaxWide + 1] = {};
+  int64_t wide_inner_launches[kMaxWide + 1] = {}, wide_sweeps_launches[kMaxWide + 1] = {};
+  std::vector<double> rhs_iters;  // inner iterations of the last reduced solves, per right-hand side
   // guess and first reduced solution
   double* guess = nullptr;
   bool has_guess = false;
@@ -280,8 +294,8 @@ struct ddps_handle {
   // CUDA graphs: launch sequences that repeat unchanged are captured once on
   // a stream of the handle and replayed (not while profiling is on)
   cudaStream_t gstream = nullptr;
-  cudaGraphExec_t g_inner = nullptr, g_factor = nullptr, g_sweeps = nullptr;
-  int64_t g_inner_launches = 0, g_factor_launches = 0, g_sweeps_launches = 0;
+  cudaGraphExec_t g_factor = nullptr;
+  int64_t g_factor_launches = 0;
   bool capturing = false;  // a capture is under way: launches go into it
   struct PrecGraph {
     const double* y;
@@ -381,9 +395,9 @@ T* dupload(ddps_handle* h, const std::vector<T>& v) {
 }
 
 // Chunk table of a segmented vector.
-SegView make_segview(ddps_handle* h, const std::vector<int64_t>& seg_ptr) {
+SegView make_segview(ddps_handle* h, const std::vector<int64_t>& seg_ptr, int64_t total = -1) {
   // chunk length: about eight chunks per SM over the whole vector, between 256 and 8192
-  const int64_t total = seg_ptr.empty() ? 0 : seg_ptr.back() - seg_ptr.front();
+  if (total < 0) total = seg_ptr.empty() ? 0 : seg_ptr.back() - seg_ptr.front();
   const int64_t CH = std::min<int64_t>(8192, std::max<int64_t>(256, (total / (8 * 152) + 255) / 256 * 256));
   std::vector<int64_t> cb, ce;
   std::vector<int32_t> cs, scp;
@@ -802,11 +816,13 @@ template <typename T>
 void sweep_launches(ddps_handle* h, T* w, T* u, cudaStream_t s) {
   const Analysis& A = h->A;
   const T* arena = (const T*)h->arena;
-  const int top = h->use_persist ? h->persist_L : A.nlevels;
+  const int nv = w == (T*)h->w ? h->width : 1;
+  const bool persist = h->use_persist && nv == 1;
+  const int top = persist ? h->persist_L : A.nlevels;
   const int64_t nf = (int64_t)A.f_k.size();
   int32_t* done_f = h->p_flags;
   int32_t* done_b = h->p_flags + nf;
-  if (h->use_persist) {
+  if (persist) {
     CK(cudaMemsetAsync(h->p_flags, 0, (2 * nf + 2) * sizeof(int32_t), s));
     launch_fwd_persist<T>(h->F, h->p_fwd, h->persist_n, h->persist_max_m, arena, w, u, done_f,
                           h->p_flags + 2 * nf, h->derr, s);
@@ -814,11 +830,13 @@ void sweep_launches(ddps_handle* h, T* w, T* u, cudaStream_t s) {
   }
   for (int L = top - 1; L >= 0; --L)
     launch_fwd1<T>(h->F, h->level_fronts + A.level_ptr[L], A.level_ptr[L + 1] - A.level_ptr[L],
-                   h->split[L].max_m, arena, w, u, s, h->tune_fwd.empty() ? SOLVE_AUTO : h->tune_fwd[L]);
+                   h->split[L].max_m, arena, w, u, s, h->tune_fwd.empty() ? SOLVE_AUTO : h->tune_fwd[L], nv,
+                   A.n, A.upd_size);
   for (int L = 0; L < top; ++L)
     launch_bwd1<T>(h->F, h->level_fronts + A.level_ptr[L], A.level_ptr[L + 1] - A.level_ptr[L],
-                   h->split[L].max_m, arena, w, s, h->tune_bwd.empty() ? SOLVE_AUTO : h->tune_bwd[L]);
-  if (h->use_persist) {
+                   h->split[L].max_m, arena, w, s, h->tune_bwd.empty() ? SOLVE_AUTO : h->tune_bwd[L], nv,
+                   A.n);
+  if (persist) {
     launch_bwd_persist<T>(h->F, h->p_bwd, h->persist_n, h->persist_max_m, h->p_wait, arena, w,
                           done_b, h->p_flags + 2 * nf + 1, h->derr, s);
     h->launches++;
@@ -841,7 +859,8 @@ void block_solve_impl(ddps_handle* h, const double* y, double* g, cudaStream_t s
     h->launches++;
     return;
   }
-  launch_permute_in<T>(y, h->perm, A.n, w, s);
+  const int nv = w == (T*)h->w ? h->width : 1;  // the handle's work vectors: of every right-hand side
+  launch_permute_in<T>(y, h->perm, A.n, w, s, nv);
   if (A.ilu) {  // (L~ U~)^-1 y: level-scheduled triangular solves
     const T* a = (const T*)h->il_val;
     for (size_t l = 0; l + 1 < A.il_lf_ptr.size(); ++l)
@@ -865,7 +884,7 @@ void block_solve_impl(ddps_handle* h, const double* y, double* g, cudaStream_t s
   } else {
     sweep_launches<T>(h, w, u, s);
   }
-  launch_permute_out<T>(w, h->perm, A.n, g, s);
+  launch_permute_out<T>(w, h->perm, A.n, g, s, nv);
   h->launches += 2;
 }
 
@@ -1090,7 +1109,13 @@ void ghat_matvec(ddps_handle* h, const TI* v, TI* w, cudaStream_t s, const KScal
     h->launches += 2;
     return;
   }
-  if (ghat_tiled<TG>(h)) {
+  if (h->width > 1) {
+    if constexpr (!std::is_same<TG, double>::value)
+      launch_ghat_matvec_multi<TG, TI>((const TG*)h->ghat, h->mv_block, h->mv_row, h->mv_h, h->mv_ntiles,
+                                       h->mv_max_cols, h->gq0, h->gq1, h->gcol_ptr, h->ghat_off, h->gld,
+                                       h->gcols, v, w, (int64_t)h->A.c.size(), h->width, h->A.nsys, sc,
+                                       h->block_sys, s);
+  } else if (ghat_tiled<TG>(h)) {
     // every block owning reduced rows has tiles (a block without coupling
     // columns gets w = v on its rows)
     launch_ghat_matvec_tiled<TG, TI>((const TG*)h->ghat, h->mv_block, h->mv_row, h->mv_h, h->mv_ntiles,
@@ -1131,7 +1156,7 @@ RedSpec nored() { return RedSpec{nullptr, nullptr, 0, 0, nullptr}; }
 template <typename TG, typename TI>
 double inner_solve(ddps_handle* h, const double* ghat64, double* zhat64, const double* z0,
                    cudaStream_t s, bool masked) {
-  const int64_t m = (int64_t)h->A.c.size();
+  const int64_t m = (int64_t)h->A.c.size() * h->width;
   const SegView& S = h->Sm;
   const int ns = h->nseg;
   KScal* sc = h->sc_in;
@@ -1141,7 +1166,7 @@ double inner_solve(ddps_handle* h, const double* ghat64, double* zhat64, const d
     explicit HostScalars(ddps_handle* hh) : h(hh), saved(hh->hsc) { h->hsc = h->hsc_in; }
     ~HostScalars() { h->hsc = saved; }
   } host_scalars(h);
-  if (h->inner.ok) {  // every system fits the shared memory of a cluster
+  if (h->inner.ok && h->width == 1) {  // every system fits the shared memory of a cluster
     {
       Prof pr(h, DDPS_PROF_GHAT_MATVEC, s);
       h->launches += launch_inner_cluster<TG, TI>(h->inner, (const TG*)h->ghat, ghat64, z0, zhat64,
@@ -1224,7 +1249,7 @@ double inner_solve(ddps_handle* h, const double* ghat64, double* zhat64, const d
   // one BiCGStab iteration; `it` < 0: the iteration number lives on the device
   // with the tiled G^ product, sigma and (t, s), (t, t) are reduced by the
   // products themselves, which also take the alpha and omega steps
-  const bool fold = ghat_tiled<TG>(h);
+  const bool fold = ghat_tiled<TG>(h) && h->width == 1;
   auto iteration = [&](int it, cudaStream_t st) {
     update_p<TI>(S, sc, r, p, v, st);
     if (fold) {
@@ -1308,6 +1333,11 @@ double inner_solve(ddps_handle* h, const double* ghat64, double* zhat64, const d
   for (double v2 : iters) mx = std::max(mx, v2);
   for (int q = 0; q < ns; ++q)
     if (h->hsc[q].active) mx = std::max(mx, (double)h->opt.maxit_in);
+  h->rhs_iters.assign(h->width, 0.0);
+  for (int q = 0; q < ns; ++q) {
+    double& it = h->rhs_iters[q / h->A.nsys];
+    it = std::max(it, h->hsc[q].active ? (double)h->opt.maxit_in : iters[q]);
+  }
   return mx;
 }
 
@@ -1366,21 +1396,39 @@ void precond_apply(ddps_handle* h, const double* y, double* z, cudaStream_t s, b
     h->stat_precond++;
     return;
   }
-  launch_gather(h->pc_g, h->c, m, h->pc_ghat, s);                        // 6.2
-  h->launches++;
+  const int nv = h->width;
+  for (int r = 0; r < nv; ++r)
+    launch_gather(h->pc_g + r * h->A.n, h->c, m, h->pc_ghat + r * m, s);  // 6.2
+  h->launches += nv;
   const double* z0 = (first && h->has_guess) ? h->guess : nullptr;
   const double its = inner_dispatch(h, h->pc_ghat, h->pc_zhat, z0, s, masked);  // 6.3
-  h->stat_inner += (int64_t)std::ceil(its);
+  int last = 0, applied = 1;
+  if (nv == 1) {
+    h->stat_inner += (int64_t)std::ceil(its);
+    if (first) h->stat_first_inner = its;
+  } else {  // counted for the right-hand sides that are still iterated
+    applied = 0;
+    for (int r = 0; r < nv; ++r) {
+      bool active = false;
+      for (int q = 0; q < h->A.nsys; ++q) active |= h->hsc_out[r * h->A.nsys + q].active != 0;
+      if (!active) continue;
+      h->stat_inner += (int64_t)std::ceil(h->rhs_iters[r]);
+      if (first && r == 0) h->stat_first_inner = h->rhs_iters[0];
+      last = r;
+      ++applied;
+    }
+  }
   if (first) {
-    h->stat_first_inner = its;
-    CK(cudaMemcpyAsync(h->first_zhat, h->pc_zhat, m * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    CK(cudaMemcpyAsync(h->first_ghat, h->pc_ghat, m * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    CK(cudaMemcpyAsync(h->first_zhat, h->pc_zhat + last * m, m * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    CK(cudaMemcpyAsync(h->first_ghat, h->pc_ghat + last * m, m * sizeof(double), cudaMemcpyDeviceToDevice, s));
   }
   // 6.4-6.5: z = g - G(:,c) z^ = D~^-1 (y - R~ z^)
-  launch_rt_residual(h->rt_rowptr, h->rt_col, h->rt_val, h->A.n, y, h->pc_zhat, h->pc_t, s, h->tune_rt);
-  h->launches++;
+  for (int r = 0; r < nv; ++r)
+    launch_rt_residual(h->rt_rowptr, h->rt_col, h->rt_val, h->A.n, y + r * h->A.n, h->pc_zhat + r * m,
+                       h->pc_t + r * h->A.n, s, h->tune_rt);
+  h->launches += nv;
   block_solve(h, h->pc_t, z, s);
-  h->stat_precond++;
+  h->stat_precond += applied;
 }
 
 void precond_direct_launches(ddps_handle* h, const double* y, double* z, cudaStream_t s) {
@@ -1405,14 +1453,15 @@ void precond_direct_launches(ddps_handle* h, const double* y, double* z, cudaStr
 ddps_status solve_impl(ddps_handle* h, const double* f, double* x, const double* x0,
                        cudaStream_t s, ddps_solve_info* info) {
   const Analysis& A = h->A;
-  const int64_t n = A.n;
+  const int64_t n = A.n * h->width;
   const SegView& S = h->Sn;
   const int ns = h->nseg;
   KScal* sc = h->sc_out;
   auto spmv = [&](const double* in, double* out) {
     Prof pr(h, DDPS_PROF_SPMV, s);
-    launch_spmv(h->rowptr, h->colind, h->vals, n, in, out, s, h->tune_spmv);
-    h->launches++;
+    for (int r = 0; r < h->width; ++r)
+      launch_spmv(h->rowptr, h->colind, h->vals, A.n, in + r * A.n, out + r * A.n, s, h->tune_spmv);
+    h->launches += h->width;
   };
   h->stat_inner = 0;
   h->stat_precond = 0;
@@ -1584,6 +1633,107 @@ ddps_status solve_impl(ddps_handle* h, const double* f, double* x, const double*
   }
   return DDPS_OK;
 }
+
+// Several right-hand sides are iterated together when the passes over G^ dominate: with an
+// iterative reduced solve on a stored G^ of at most 32 bits (an FP64 product is bound by the
+// FP64 pipe, not by memory; systems that fit a cluster have their own launch).  Four right-hand
+// sides, 48^3 in eight slabs, FP16 G^: G^ products 14.0 -> 4.5 ms, block solves (the vectors
+// in the grid's second dimension) 4.7 -> 2.9, launches 1,484 -> 476, the solve 22.9 -> 10.0.
+int wide_width(ddps_handle* h, int32_t nrhs) {
+  const Analysis& A = h->A;
+  if (nrhs < 2 || A.c.empty() || A.ilu || h->use_direct || h->inner.ok || h->has_guess || h->wide_failed ||
+      h->opt.ghat_mode == DDPS_GHAT_IMPLICIT || h->opt.ghat_prec == DDPS_FP64)
+    return 1;
+  int W = std::min<int32_t>(nrhs, kMaxWide);
+  while (W > 1 && ghat_multi_smem(h->mv_max_cols, W) > 200 * 1024) --W;
+  return W;
+}
+
+constexpr int64_t kWideBytes = (int64_t)4 << 30;  // most memory taken for the wide vectors
+
+// The wide workspace, in one allocation; false if it is too large or there is no room.
+bool ensure_wide(ddps_handle* h) {
+  if (h->wide_ok) return true;
+  const Analysis& A = h->A;
+  const int64_t W = kMaxWide, n = A.n, m = (int64_t)A.c.size(), ns = A.nsys * W;
+  const int64_t fs = (int64_t)prec_size(h->opt.factor_prec), is = (int64_t)prec_size(h->opt.inner_prec);
+  auto up = [](int64_t b) { return (b + 255) / 256 * 256; };
+  const int64_t bn = up(W * n * 8), bm = up(W * m * 8), bi = up(W * m * is), bw = up(W * n * fs),
+                bu = up(W * std::max<int64_t>(A.upd_size, 1) * fs);
+  const int64_t total = 12 * bn + 2 * bm + 8 * bi + bw + bu;
+  SolveWork& k = h->wide;
+  if (total > kWideBytes) {
+    h->wide_failed = true;
+    return false;
+  }
+  try {
+    char* p = (char*)dalloc_bytes(h, total);
+    auto take = [&](int64_t b) {
+      char* q = p;
+      p += b;
+      return (void*)q;
+    };
+    double** outer[] = {&k.o_r, &k.o_rhat, &k.o_p, &k.o_v, &k.o_phat, &k.o_s,
+                        &k.o_shat, &k.o_t, &k.o_xt, &k.o_tmp, &k.pc_g, &k.pc_t};
+    for (double** pp : outer) *pp = (double*)take(bn);
+    k.pc_ghat = (double*)take(bm);
+    k.pc_zhat = (double*)take(bm);
+    void** inner[] = {&k.i_g, &k.i_z, &k.i_r, &k.i_rh, &k.i_p, &k.i_v, &k.i_s, &k.i_t};
+    for (void** pp : inner) *pp = take(bi);
+    k.w = take(bw);
+    k.updv = take(bu);
+    std::vector<int64_t> pn, pm;
+    for (int r = 0; r < W; ++r)
+      for (int32_t q = 0; q < A.nsys; ++q) {
+        pn.push_back(r * n + A.sys_row_ptr[q]);
+        pm.push_back(r * m + A.sys_c_ptr[q]);
+      }
+    pn.push_back(W * n);
+    pm.push_back(W * m);
+    k.Sn = make_segview(h, pn, n);  // chunks, and so sums, as for a single right-hand side
+    k.Sm = make_segview(h, pm, m);
+    k.sc_out = dalloc<KScal>(h, ns);
+    k.sc_in = dalloc<KScal>(h, ns);
+    k.partial = dalloc<double>(h, 3 * (int64_t)std::max(k.Sn.nchunks, k.Sm.nchunks) + 3);
+    CK(cudaMallocHost((void**)&k.hsc_out, sizeof(KScal) * ns));
+    CK(cudaMallocHost((void**)&k.hsc_in, sizeof(KScal) * ns));
+    CK(cudaMallocHost((void**)&k.hstage, sizeof(KScal) * ns * kStageSlots));
+    k.hsc = k.hsc_out;
+  } catch (const Fail&) {  // one after the other then
+    cudaGetLastError();
+    h->wide_failed = true;
+    return false;
+  }
+  h->wide_ok = true;
+  return true;
+}
+
+// Puts the wide workspace, cut to W right-hand sides, in the place of the handle's.
+struct WideScope {
+  ddps_handle* h;
+  SolveWork saved;
+  int W;
+  WideScope(ddps_handle* hh, int w) : h(hh), saved(*hh), W(w) {
+    SolveWork k = h->wide;
+    k.width = W;
+    k.nseg = W * h->A.nsys;
+    k.Sn.nseg = k.Sm.nseg = k.nseg;
+    k.Sn.nchunks = k.Sn.nchunks / kMaxWide * W;
+    k.Sm.nchunks = k.Sm.nchunks / kMaxWide * W;
+    k.g_inner = h->wide_inner[W];
+    k.g_inner_launches = h->wide_inner_launches[W];
+    k.g_sweeps = h->wide_sweeps[W];
+    k.g_sweeps_launches = h->wide_sweeps_launches[W];
+    static_cast<SolveWork&>(*h) = k;
+  }
+  ~WideScope() {
+    h->wide_inner[W] = h->g_inner;
+    h->wide_inner_launches[W] = h->g_inner_launches;
+    h->wide_sweeps[W] = h->g_sweeps;
+    h->wide_sweeps_launches[W] = h->g_sweeps_launches;
+    static_cast<SolveWork&>(*h) = saved;
+  }
+};
 
 ddps_status fail(ddps_handle* h, const Fail& e) {
   if (h) h->err = e.msg;
@@ -2583,9 +2733,16 @@ ddps_status ddps_solve(ddps_handle* h, const double* f, double* x, int32_t nrhs,
     const int64_t n = h->A.n;
     ddps_status worst = DDPS_OK;
     ddps_solve_info acc{}, one{};
-    for (int32_t j = 0; j < nrhs; ++j) {
-      ddps_status st = solve_impl(h, f + j * n, x + j * n, x0 ? x0 + j * n : nullptr,
-                                  as_stream(stream), &one);
+    for (int32_t j = 0, W = 1; j < nrhs; j += W) {
+      W = wide_width(h, nrhs - j);
+      if (W > 1 && !ensure_wide(h)) W = 1;
+      ddps_status st;
+      if (W > 1) {
+        WideScope scope(h, W);
+        st = solve_impl(h, f + j * n, x + j * n, x0 ? x0 + j * n : nullptr, as_stream(stream), &one);
+      } else {
+        st = solve_impl(h, f + j * n, x + j * n, x0 ? x0 + j * n : nullptr, as_stream(stream), &one);
+      }
       merge_info(&acc, one, j == 0);
       if (st != DDPS_OK) worst = st;
     }
@@ -2898,6 +3055,13 @@ ddps_status ddps_destroy(ddps_handle* h) {
   if (h->hsc_out) cudaFreeHost(h->hsc_out);
   if (h->hsc_in) cudaFreeHost(h->hsc_in);
   if (h->hstage) cudaFreeHost(h->hstage);
+  if (h->wide.hsc_out) cudaFreeHost(h->wide.hsc_out);
+  if (h->wide.hsc_in) cudaFreeHost(h->wide.hsc_in);
+  if (h->wide.hstage) cudaFreeHost(h->wide.hstage);
+  for (int W = 2; W <= kMaxWide; ++W) {
+    if (h->wide_inner[W]) cudaGraphExecDestroy(h->wide_inner[W]);
+    if (h->wide_sweeps[W]) cudaGraphExecDestroy(h->wide_sweeps[W]);
+  }
   if (h->any_host) cudaFreeHost(h->any_host);
   delete h;
   return DDPS_OK;

@@ -273,9 +273,11 @@ void launch_ghat_extract(const int32_t* qblock, const int32_t* c_rownew, const i
 
 // ---- solve.cu ---------------------------------------------------------------
 template <typename T>
-void launch_permute_in(const double* y, const int32_t* perm, int64_t n, T* w, cudaStream_t s);
+void launch_permute_in(const double* y, const int32_t* perm, int64_t n, T* w, cudaStream_t s,
+                       int nv = 1);  // nv vectors, n entries apart
 template <typename T>
-void launch_permute_out(const T* w, const int32_t* perm, int64_t n, double* g, cudaStream_t s);
+void launch_permute_out(const T* w, const int32_t* perm, int64_t n, double* g, cudaStream_t s,
+                        int nv = 1);
 // Launch shapes of a block-solve depth (see launch_fwd1): automatic, one warp
 // per front, one CTA per front with eight loads in flight per lane, or a
 // cluster of 1, 2, 4 or 8 CTAs per front with thirty-two.
@@ -285,10 +287,11 @@ inline int solve_cfg_cluster(int c) { return c >= 8 ? SOLVE_CL8 : c >= 4 ? SOLVE
 inline int solve_cfg_size(int cfg) { return cfg == SOLVE_CL8 ? 8 : cfg == SOLVE_CL4 ? 4 : cfg == SOLVE_CL2 ? 2 : 1; }
 template <typename T>
 void launch_fwd1(DevFronts F, const int32_t* list, int32_t nf, int32_t max_m, const T* arena,
-                 T* w, T* u, cudaStream_t s, int cfg = SOLVE_AUTO);
+                 T* w, T* u, cudaStream_t s, int cfg = SOLVE_AUTO, int nv = 1, int64_t wst = 0,
+                 int64_t ust = 0);  // nv vectors, wst and ust entries apart
 template <typename T>
 void launch_bwd1(DevFronts F, const int32_t* list, int32_t nf, int32_t max_m, const T* arena,
-                 T* w, cudaStream_t s, int cfg = SOLVE_AUTO);
+                 T* w, cudaStream_t s, int cfg = SOLVE_AUTO, int nv = 1, int64_t wst = 0);
 // CSR product kernels (the autotuner picks per matrix): row blocks streamed
 // through shared memory (SPMV_BLOCK: all of a thread's loads of the block
 // issued at once, 16-byte vectors), 4 / 8 lanes per row, or 32-row groups
@@ -324,6 +327,17 @@ void launch_ghat_matvec_tiled(const TG* ghat, const int32_t* tile_block, const i
                               const int64_t* gld, const int32_t* gcols, const TI* v, TI* w,
                               const KScal* sc, const int32_t* block_sys, const MvRed* red,
                               cudaStream_t s);
+// w = v + G^ v for nv = 2 to 4 vectors, m entries apart (sc: nv x nsys); not for FP64 G^.
+inline size_t ghat_multi_smem(int64_t max_cols, int nv) {
+  return (size_t)(nv > 2 ? 4 : 2) * (size_t)((max_cols + 7) / 8 * 8) * sizeof(float);
+}
+template <typename TG, typename TI>
+void launch_ghat_matvec_multi(const TG* ghat, const int32_t* tile_block, const int32_t* tile_row,
+                              const int32_t* tile_h, int32_t ntiles, int64_t max_cols,
+                              const int64_t* gq0, const int64_t* gq1, const int64_t* gcol_ptr,
+                              const int64_t* ghat_off, const int64_t* gld, const int32_t* gcols,
+                              const TI* v, TI* w, int64_t m, int nv, int nsys, const KScal* sc,
+                              const int32_t* block_sys, cudaStream_t s);
 void launch_gather(const double* src, const int64_t* idx, int64_t m, double* dst, cudaStream_t s);
 void launch_gather_rt_values(const double* values, const int64_t* rt_src, int64_t nrt,
                              double* rt_val, cudaStream_t s);

@@ -27,6 +27,8 @@ inline int grid_for(int64_t work, int threads, int cap = 152 * 32) {
 template <typename T>
 __global__ void k_permute_in(const double* __restrict__ y, const int32_t* __restrict__ perm,
                              int64_t n, T* __restrict__ w) {
+  y += blockIdx.y * n;  // one of several vectors
+  w += blockIdx.y * n;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     w[i] = (T)y[perm[i]];
@@ -35,6 +37,8 @@ __global__ void k_permute_in(const double* __restrict__ y, const int32_t* __rest
 template <typename T>
 __global__ void k_permute_out(const T* __restrict__ w, const int32_t* __restrict__ perm, int64_t n,
                               double* __restrict__ g) {
+  w += blockIdx.y * n;
+  g += blockIdx.y * n;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     g[perm[i]] = (double)w[i];
@@ -178,8 +182,10 @@ constexpr int kMaxChildren = 16;
 template <typename T, int NT, int CH, int NSEG, int B>
 __global__ void __launch_bounds__(NT, B == 8 ? 8 : 2)
     k_fwd1(DevFronts F, const int32_t* __restrict__ list, const T* __restrict__ arena,
-           T* __restrict__ w, T* __restrict__ u) {
+           T* __restrict__ w, T* __restrict__ u, int64_t wst, int64_t ust) {
   extern __shared__ unsigned char smem_raw[];
+  w += blockIdx.y * wst;  // one of several vectors
+  u += blockIdx.y * ust;
   T* red = reinterpret_cast<T*>(smem_raw);  // NSEG x CH entries
   T* t = red + NSEG * CH;                   // m entries
   __shared__ int32_t ch_rc[kMaxChildren];
@@ -245,8 +251,9 @@ __global__ void __launch_bounds__(NT, B == 8 ? 8 : 2)
 template <typename T, int NT, int CH, int NSEG, int B>
 __global__ void __launch_bounds__(NT, B == 8 ? 8 : 2)
     k_bwd1(DevFronts F, const int32_t* __restrict__ list, const T* __restrict__ arena,
-           T* __restrict__ w) {
+           T* __restrict__ w, int64_t wst) {
   extern __shared__ unsigned char smem_raw[];
+  w += blockIdx.y * wst;
   T* red = reinterpret_cast<T*>(smem_raw);  // NSEG x CH entries
   T* t = red + NSEG * CH;                   // k entries, then x_upd (r entries)
   pdl_trigger();
@@ -309,8 +316,10 @@ __device__ __forceinline__ T warp_row_dot(const T* __restrict__ Ai, int64_t m, i
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
     k_fwd1w(DevFronts F, const int32_t* __restrict__ list, int32_t nf, int32_t ldt,
-            const T* __restrict__ arena, T* __restrict__ w, T* __restrict__ u) {
+            const T* __restrict__ arena, T* __restrict__ w, T* __restrict__ u, int64_t wst, int64_t ust) {
   extern __shared__ unsigned char smem_raw[];
+  w += blockIdx.y * wst;
+  u += blockIdx.y * ust;
   pdl_trigger();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = blockIdx.x * (kThreads / 32) + warp;
@@ -347,8 +356,9 @@ __global__ void __launch_bounds__(kThreads)
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
     k_bwd1w(DevFronts F, const int32_t* __restrict__ list, int32_t nf, int32_t ldt,
-            const T* __restrict__ arena, T* __restrict__ w) {
+            const T* __restrict__ arena, T* __restrict__ w, int64_t wst) {
   extern __shared__ unsigned char smem_raw[];
+  w += blockIdx.y * wst;
   pdl_trigger();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = blockIdx.x * (kThreads / 32) + warp;
@@ -1040,13 +1050,108 @@ __global__ void k_gather(const double* __restrict__ src, const int64_t* __restri
 
 }  // namespace
 
+// The same product with up to R vectors (m entries apart) in one pass over G^: a single
+// vector's is bound by the bytes of G^ (85% of the copy bandwidth), so several right-hand
+// sides at once cost little more than one.  16 warps, each four rows at once; the vectors'
+// coupling entries in shared memory, one after the other (16-byte reads); a row's sum for a
+// vector takes the order of the single product.  Vectors past nv repeat the last one.
+// 48^3, eight slabs, FP16 G^ (276 MB): four vectors 62 us, one 49.
+constexpr int kMultiThreads = 512;
+template <typename TG, typename TI, int R>
+__global__ void __launch_bounds__(kMultiThreads)
+    k_ghat_matvec_multi(const TG* __restrict__ ghat, const int32_t* __restrict__ tile_block,
+                        const int32_t* __restrict__ tile_row, const int32_t* __restrict__ tile_h,
+                        const int64_t* __restrict__ gq0, const int64_t* __restrict__ gq1,
+                        const int64_t* __restrict__ gcol_ptr, const int64_t* __restrict__ ghat_off,
+                        const int64_t* __restrict__ gld, const int32_t* __restrict__ gcols,
+                        const TI* __restrict__ v, TI* __restrict__ w, int64_t m, int nv, int nsys,
+                        const KScal* __restrict__ sc, const int32_t* __restrict__ block_sys) {
+  constexpr int VN = Vec16<TG>::n;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float* xs = reinterpret_cast<float*>(smem_raw);
+  const int32_t b = tile_block[blockIdx.x];
+  bool live = !sc;
+  for (int r = 0; r < nv && !live; ++r) live = sc[(int64_t)r * nsys + block_sys[b]].active;
+  if (!live) return;  // this system's inner solves have stopped
+  const int64_t r0 = tile_row[blockIdx.x];
+  const int64_t c0 = gcol_ptr[b];
+  const int nc = (int)(gcol_ptr[b + 1] - c0), ncp = (nc + 7) / 8 * 8;
+  const int64_t nrows = gq1[b] - gq0[b];
+  for (int j = threadIdx.x; j < nc; j += kMultiThreads) {
+    const int64_t c = gcols[c0 + j];
+#pragma unroll
+    for (int r = 0; r < R; ++r) xs[r * ncp + j] = (float)v[min(r, nv - 1) * m + c];
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const TG* __restrict__ base = ghat + ghat_off[b];
+  const int nvec = nc / VN;
+  const int64_t ld = gld[b], q0 = gq0[b];
+  const int th = tile_h[blockIdx.x];
+  for (int rr = warp * 4; rr < th; rr += kMultiThreads / 32 * 4) {
+    const int64_t ra = r0 + rr;
+    if (ra >= nrows) break;
+    const int na = (int)min((int64_t)4, nrows - ra);
+    const TG* __restrict__ p[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) p[u] = base + (ra + min(u, na - 1)) * ld;
+    float acc[R][4];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) acc[r][u] = 0.f;
+#pragma unroll 2
+    for (int q = lane; q < nvec; q += 32) {
+      float g[4][VN];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) load16<TG>(p[u] + q * VN, g[u]);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        float x[VN];
+#pragma unroll
+        for (int e = 0; e < VN; e += 4)
+          *reinterpret_cast<float4*>(x + e) = *reinterpret_cast<const float4*>(xs + r * ncp + q * VN + e);
+#pragma unroll
+        for (int e = 0; e < VN; ++e)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) acc[r][u] += g[u][e] * x[e];
+      }
+    }
+    for (int j = nvec * VN + lane; j < nc; j += 32) {  // ragged tail
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float gv = to_acc<float>(p[u][j]);
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r][u] += gv * xs[r * ncp + j];
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc[r][u] += __shfl_xor_sync(0xffffffffu, acc[r][u], o);
+    if (lane == 0) {
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        if (r < nv)
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (u < na) {
+              const int64_t q = r * m + q0 + ra + u;
+              w[q] = (TI)((float)v[q] + acc[r][u]);
+            }
+    }
+  }
+}
+
 template <typename T>
-void launch_permute_in(const double* y, const int32_t* perm, int64_t n, T* w, cudaStream_t s) {
-  k_permute_in<T><<<grid_for(n, kThreads), kThreads, 0, s>>>(y, perm, n, w);
+void launch_permute_in(const double* y, const int32_t* perm, int64_t n, T* w, cudaStream_t s, int nv) {
+  k_permute_in<T><<<dim3((unsigned)grid_for(n, kThreads), nv), kThreads, 0, s>>>(y, perm, n, w);
 }
 template <typename T>
-void launch_permute_out(const T* w, const int32_t* perm, int64_t n, double* g, cudaStream_t s) {
-  k_permute_out<T><<<grid_for(n, kThreads), kThreads, 0, s>>>(w, perm, n, g);
+void launch_permute_out(const T* w, const int32_t* perm, int64_t n, double* g, cudaStream_t s, int nv) {
+  k_permute_out<T><<<dim3((unsigned)grid_for(n, kThreads), nv), kThreads, 0, s>>>(w, perm, n, g);
 }
 
 static int sm_count() { return device_sm_count(); }
@@ -1057,13 +1162,13 @@ static int sm_count() { return device_sm_count(); }
 // per front, within two CTAs per SM (always eight for very large fronts),
 // and kSolveB loads per lane.
 template <typename K, typename... Args>
-static void launch_clustered(K kern, int32_t nf, int c, size_t sm, cudaStream_t s, Args... args) {
+static void launch_clustered(K kern, int32_t nf, int nv, int c, size_t sm, cudaStream_t s, Args... args) {
   // the 48 KB that need no opt-in hold the kernel's static shared memory too
   if (sm > 40 * 1024)
     record_launch_error(
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(nf * c));
+  cfg.gridDim = dim3((unsigned)(nf * c), (unsigned)nv);
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = sm;
   cfg.stream = s;
@@ -1109,7 +1214,7 @@ static bool warp_solve_level(int32_t nf, int32_t max_m) {
 // flight per lane for many fronts, else clusters); the autotuner may fix it.
 template <typename T>
 void launch_fwd1(DevFronts F, const int32_t* list, int32_t nf, int32_t max_m, const T* arena,
-                 T* w, T* u, cudaStream_t s, int cfg) {
+                 T* w, T* u, cudaStream_t s, int cfg, int nv, int64_t wst, int64_t ust) {
   if (nf <= 0) return;
   if (cfg == SOLVE_AUTO)
     cfg = warp_solve_level(nf, max_m) ? SOLVE_WARP
@@ -1119,19 +1224,19 @@ void launch_fwd1(DevFronts F, const int32_t* list, int32_t nf, int32_t max_m, co
     const int32_t ldt = 2 * max_m;
     const size_t smw = (size_t)(kThreads / 32) * ldt * sizeof(T);
     const int32_t grid = (nf + kThreads / 32 - 1) / (kThreads / 32);
-    launch_clustered(k_fwd1w<T>, grid, 1, smw, s, F, list, nf, ldt, arena, w, u);
+    launch_clustered(k_fwd1w<T>, grid, nv, 1, smw, s, F, list, nf, ldt, arena, w, u, wst, ust);
     return;
   }
   if (cfg == SOLVE_CTA8)
-    launch_clustered(k_fwd1<T, kThreads, kSolveCh, 8, 8>, nf, 1,
-                     ((size_t)2 * max_m + kSolveRed) * sizeof(T), s, F, list, arena, w, u);
+    launch_clustered(k_fwd1<T, kThreads, kSolveCh, 8, 8>, nf, nv, 1,
+                     ((size_t)2 * max_m + kSolveRed) * sizeof(T), s, F, list, arena, w, u, wst, ust);
   else
-    launch_clustered(k_fwd1<T, kThreads, kSolveChW, 8, kSolveB>, nf, solve_cfg_size(cfg),
-                     ((size_t)2 * max_m + kSolveRedW) * sizeof(T), s, F, list, arena, w, u);
+    launch_clustered(k_fwd1<T, kThreads, kSolveChW, 8, kSolveB>, nf, nv, solve_cfg_size(cfg),
+                     ((size_t)2 * max_m + kSolveRedW) * sizeof(T), s, F, list, arena, w, u, wst, ust);
 }
 template <typename T>
 void launch_bwd1(DevFronts F, const int32_t* list, int32_t nf, int32_t max_m, const T* arena,
-                 T* w, cudaStream_t s, int cfg) {
+                 T* w, cudaStream_t s, int cfg, int nv, int64_t wst) {
   if (nf <= 0) return;
   if (cfg == SOLVE_AUTO)
     cfg = warp_solve_level(nf, max_m) ? SOLVE_WARP
@@ -1141,15 +1246,15 @@ void launch_bwd1(DevFronts F, const int32_t* list, int32_t nf, int32_t max_m, co
     const int32_t ldt = max_m;
     const size_t smw = (size_t)(kThreads / 32) * ldt * sizeof(T);
     const int32_t grid = (nf + kThreads / 32 - 1) / (kThreads / 32);
-    launch_clustered(k_bwd1w<T>, grid, 1, smw, s, F, list, nf, ldt, arena, w);
+    launch_clustered(k_bwd1w<T>, grid, nv, 1, smw, s, F, list, nf, ldt, arena, w, wst);
     return;
   }
   if (cfg == SOLVE_CTA8)
-    launch_clustered(k_bwd1<T, kThreads, kSolveCh, 8, 8>, nf, 1,
-                     ((size_t)max_m + kSolveRed) * sizeof(T), s, F, list, arena, w);
+    launch_clustered(k_bwd1<T, kThreads, kSolveCh, 8, 8>, nf, nv, 1,
+                     ((size_t)max_m + kSolveRed) * sizeof(T), s, F, list, arena, w, wst);
   else
-    launch_clustered(k_bwd1<T, kThreads, kSolveChW, 8, kSolveB>, nf, solve_cfg_size(cfg),
-                     ((size_t)max_m + kSolveRedW) * sizeof(T), s, F, list, arena, w);
+    launch_clustered(k_bwd1<T, kThreads, kSolveChW, 8, kSolveB>, nf, nv, solve_cfg_size(cfg),
+                     ((size_t)max_m + kSolveRedW) * sizeof(T), s, F, list, arena, w, wst);
 }
 
 // Persistent sweeps: enough warps for every front, at most eight CTAs of
@@ -1244,6 +1349,34 @@ void launch_ghat_matvec(const TG* ghat, const int32_t* qblock, const int64_t* gq
 }
 
 template <typename TG, typename TI>
+void launch_ghat_matvec_multi(const TG* ghat, const int32_t* tile_block, const int32_t* tile_row,
+                              const int32_t* tile_h, int32_t ntiles, int64_t max_cols,
+                              const int64_t* gq0, const int64_t* gq1, const int64_t* gcol_ptr,
+                              const int64_t* ghat_off, const int64_t* gld, const int32_t* gcols,
+                              const TI* v, TI* w, int64_t m, int nv, int nsys, const KScal* sc,
+                              const int32_t* block_sys, cudaStream_t s) {
+  if (ntiles <= 0) return;
+  const int R = nv > 2 ? 4 : 2;
+  const size_t sm = ghat_multi_smem(max_cols, nv);
+  auto k = R == 4 ? k_ghat_matvec_multi<TG, TI, 4> : k_ghat_matvec_multi<TG, TI, 2>;
+  if (sm > 40 * 1024)  // static bytes count too
+    record_launch_error(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  k<<<ntiles, kMultiThreads, sm, s>>>(ghat, tile_block, tile_row, tile_h, gq0, gq1, gcol_ptr, ghat_off,
+                                      gld, gcols, v, w, m, nv, nsys, sc, block_sys);
+}
+#define DDPS_INST_MM(TG, TI)                                                                      \
+  template void launch_ghat_matvec_multi<TG, TI>(                                                 \
+      const TG*, const int32_t*, const int32_t*, const int32_t*, int32_t, int64_t, const int64_t*, \
+      const int64_t*, const int64_t*, const int64_t*, const int64_t*, const int32_t*, const TI*, TI*, \
+      int64_t, int, int, const KScal*, const int32_t*, cudaStream_t);
+DDPS_INST_MM(float, double)
+DDPS_INST_MM(float, float)
+DDPS_INST_MM(__half, double)
+DDPS_INST_MM(__half, float)
+DDPS_INST_MM(__nv_bfloat16, double)
+DDPS_INST_MM(__nv_bfloat16, float)
+
+template <typename TG, typename TI>
 void launch_ghat_matvec_tiled(const TG* ghat, const int32_t* tile_block, const int32_t* tile_row,
                               const int32_t* tile_h, int32_t ntiles, int64_t max_cols,
                               const int64_t* gq0,
@@ -1283,12 +1416,14 @@ DDPS_INST_P(double)
 DDPS_INST_P(float)
 
 #define DDPS_INST_S(T)                                                                          \
-  template void launch_permute_in<T>(const double*, const int32_t*, int64_t, T*, cudaStream_t); \
-  template void launch_permute_out<T>(const T*, const int32_t*, int64_t, double*, cudaStream_t);\
+  template void launch_permute_in<T>(const double*, const int32_t*, int64_t, T*, cudaStream_t,  \
+                                     int);                                                      \
+  template void launch_permute_out<T>(const T*, const int32_t*, int64_t, double*, cudaStream_t, \
+                                      int);                                                     \
   template void launch_fwd1<T>(DevFronts, const int32_t*, int32_t, int32_t, const T*, T*, T*,   \
-                               cudaStream_t, int);                                              \
+                               cudaStream_t, int, int, int64_t, int64_t);                       \
   template void launch_bwd1<T>(DevFronts, const int32_t*, int32_t, int32_t, const T*, T*,       \
-                               cudaStream_t, int);
+                               cudaStream_t, int, int, int64_t);
 DDPS_INST_S(double)
 DDPS_INST_S(float)
 
