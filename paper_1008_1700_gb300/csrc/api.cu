@@ -2249,7 +2249,7 @@ void build_device(ddps_handle* h, const int32_t* rowptr, const int32_t* colind) 
     {
       const int64_t bytes = std::max<int64_t>(inv_total, 1) * (int64_t)prec_size(h->opt.factor_prec);
       h->inv = dalloc_bytes(h, bytes);
-      CK(cudaMemset(h->inv, 0, bytes));  // the diagonal blocks' other triangles stay zero
+      CK(cudaMemset(h->inv, 0, bytes));  // the diagonal tiles' other triangles stay zero
     }
     if (h->opt.factor_prec == DDPS_FP32) build_inverse_products(h, order, ioff);
     h->lu_panel_fronts = dupload(h, pfronts);

@@ -89,12 +89,35 @@ __global__ void k_extend_add_p(DevFronts F, const int32_t* __restrict__ parent,
 constexpr int NB = 32;
 constexpr int TT = 64;
 
+// A pivot p of type T passes |p| > t exactly if |p| > threshold<T>(t): the largest T not
+// above t (an FP64 comparison in the chain of pivots costs as much as 30 FP32 operations).
+template <typename T>
+__device__ __forceinline__ T threshold(double t) {
+  if constexpr (sizeof(T) == 4)
+    return __double2float_rd(t);
+  else
+    return t;
+}
+// What a pivot that does not pass is replaced with (the factorisation fails, but finitely).
+template <typename T>
+__device__ __forceinline__ T replacement(T piv, double t) {
+  const double rep = t > 0.0 ? t : 1e-300;
+  return (T)(piv < T(0) ? -rep : rep);
+}
+// a / d from r = 1 / d, with the remainder put back: two roundings less than a r.
+template <typename T>
+__device__ __forceinline__ T quotient(T a, T d, T r) {
+  const T q = a * r, e = fma(-q, d, a);
+  return fma(e, r, q);
+}
+
 // ---------------------------------------------------------------------------
 // Large fronts, several CTAs per front: blocked right-looking LU, one panel
 // of 32 pivots at a time.  Without pivoting the panel
 // splits into independent parts: the 32 x 32 diagonal block is factored
 // first (k_lu_diag, one CTA per front, which also forms the inverses of its
-// two triangles into a scratch block per front), then every row below it
+// two triangles into a scratch block per front: one warp with a row per lane in
+// registers; through shared memory the depths of 64^3 in sixteen slabs took 4.0 ms, now 2.7), then every row below it
 // takes its L21 row as a U11^-1 and every column to the right its U12
 // column as L11^-1 a (k_lu_panel_rows, CTAs over chunks of 256 rows or
 // columns of every front of the depth), then the trailing update
@@ -115,38 +138,41 @@ __global__ void __launch_bounds__(kThreads)
   const int tid = threadIdx.x;
   const int jb = min(NB, k - j0);
   __shared__ T D[NB][NB + 1];
-  __shared__ double thr[NB];
+  __shared__ T thr[NB];
   for (int t = tid; t < NB * NB; t += blockDim.x) {
     const int r = t % NB, c = t / NB;
     D[r][c] = (r < jb && c < jb) ? A[(j0 + r) + (int64_t)(j0 + c) * m] : T(r == c ? 1 : 0);
   }
-  if (tid < jb) thr[tid] = pivot_tol * rownorm[row0 + j0 + tid];
+  if (tid < jb) thr[tid] = threshold<T>(pivot_tol * rownorm[row0 + j0 + tid]);
   __syncthreads();
   if (tid < 32) {
-    // the 32 x 32 LU by one warp: lane r owns row r of the updates
-    for (int j = 0; j < jb; ++j) {
-      T piv = D[j][j];
-      const bool small = !(fabs((double)piv) > thr[j]);
-      if (small) {
-        const double rep = thr[j] > 0.0 ? thr[j] : 1e-300;
-        piv = (T)((double)piv < 0.0 ? -rep : rep);
-      }
-      __syncwarp();  // every lane has read the pivot before it is replaced
-      if (small && tid == 0) {
-        if (atomicCAS((unsigned long long*)&err[0], 0ull, 1ull) == 0ull) {
-          err[1] = f;
-          err[2] = row0 + j0 + j;
+    // the 32 x 32 LU by one warp, lane r with row r in registers
+    T row[NB];
+#pragma unroll
+    for (int c = 0; c < NB; ++c) row[c] = D[tid][c];
+#pragma unroll
+    for (int j = 0; j < NB; ++j) {
+      T piv = __shfl_sync(0xffffffffu, row[j], j);
+      if (j < jb && !(fabs(piv) > thr[j])) {
+        piv = replacement(piv, pivot_tol * rownorm[row0 + j0 + j]);
+        if (tid == j) {
+          if (atomicCAS((unsigned long long*)&err[0], 0ull, 1ull) == 0ull) {
+            err[1] = f;
+            err[2] = row0 + j0 + j;
+          }
+          row[j] = piv;
         }
-        D[j][j] = piv;
       }
-      const T inv = T(1) / piv;
-      if (tid > j && tid < jb) {
-        const T l = D[tid][j] * inv;
-        D[tid][j] = l;
-        for (int c = j + 1; c < jb; ++c) D[tid][c] -= l * D[j][c];
+      const T l = row[j] * (T(1) / piv);
+      if (tid > j) row[j] = l;
+#pragma unroll
+      for (int c = j + 1; c < NB; ++c) {
+        const T u = __shfl_sync(0xffffffffu, row[c], j);
+        if (tid > j) row[c] -= l * u;
       }
-      __syncwarp();
     }
+#pragma unroll
+    for (int c = 0; c < NB; ++c) D[tid][c] = row[c];
   }
   __syncthreads();
   for (int t = tid; t < jb * jb; t += blockDim.x) {
@@ -160,13 +186,15 @@ __global__ void __launch_bounds__(kThreads)
   T* Li = Ui + NB * NB;
   const int lane = tid & 31, warp = tid >> 5;
   if (warp == 0) {
+    const T rinv = T(1) / D[lane][lane];
     T x[NB];
 #pragma unroll
     for (int r = NB - 1; r >= 0; --r) {
       T sacc = r == lane ? T(1) : T(0);
 #pragma unroll
       for (int p = r + 1; p < NB; ++p) sacc -= D[r][p] * x[p];
-      x[r] = r <= lane ? sacc / D[r][r] : T(0);
+      const T ri = __shfl_sync(0xffffffffu, rinv, r);
+      x[r] = r <= lane ? quotient(sacc, D[r][r], ri) : T(0);
     }
 #pragma unroll
     for (int r = 0; r < NB; ++r) Ui[r * NB + lane] = x[r];
@@ -313,6 +341,56 @@ __global__ void __launch_bounds__(kThreads)
 // ---------------------------------------------------------------------------
 constexpr int IB = 64;  // columns per CTA and rows per tile
 
+// Columns c0 .. c0 + 3 of the inverse of a triangle of the k x k block of A (shared memory,
+// column stride m; RP rows per lane) by one warp, no barriers: the columns' entries stay in
+// registers, the entry eliminated next is broadcast.  Written to G (column stride ldg; the
+// unit diagonal of a lower one too if `unit`).  rinv: reciprocals of A's diagonal (upper).
+template <typename T, int RP, bool UPPER>
+__device__ __forceinline__ void warp_tri_inverse(const T* A, const T* rinv, int m, int k, int c0, T* G,
+                                                 int64_t ldg, bool unit = false) {
+  const int lane = threadIdx.x & 31;
+  T x[4][RP];
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+#pragma unroll
+    for (int p = 0; p < RP; ++p) x[u][p] = p * 32 + lane == c0 + u ? T(1) : T(0);
+#pragma unroll
+  for (int qq = 0; qq < RP; ++qq) {
+    const int q = UPPER ? RP - 1 - qq : qq;
+    const int l0 = UPPER ? min(q * 32 + 31, min(c0 + 3, k - 1)) : max(q * 32, c0);
+    const int l1 = UPPER ? q * 32 : min(q * 32 + 31, k - 1);
+#pragma unroll 4
+    for (int l = l0; UPPER ? l >= l1 : l <= l1; l += UPPER ? -1 : 1) {
+      T xl[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        xl[u] = __shfl_sync(0xffffffffu, x[u][q], l & 31);
+        if (UPPER) {
+          xl[u] = quotient(xl[u], A[l + l * m], rinv[l]);
+          if (lane == (l & 31)) x[u][q] = xl[u];
+        }
+      }
+#pragma unroll
+      for (int p = 0; p < RP; ++p) {
+        if (UPPER ? p > q : p < q) continue;
+        const int i = p * 32 + lane;
+        const T a = (UPPER ? i < l : i > l && i < k) ? A[i + l * m] : T(0);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u][p] -= a * xl[u];
+      }
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int c = c0 + u;
+#pragma unroll
+    for (int p = 0; p < RP; ++p) {
+      const int i = p * 32 + lane;
+      if (c < k && (UPPER ? i <= c : (i > c || (unit && i == c)) && i < k)) G[i + c * ldg] = x[u][p];
+    }
+  }
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
     k_tri_inverse_diag(DevFronts F, const int32_t* __restrict__ tile_front,
@@ -326,40 +404,25 @@ __global__ void __launch_bounds__(kThreads)
   const int32_t ld = inv_ld(k);
   T* __restrict__ X = inv + inv_off[f] + (upper ? (int64_t)ld * k : 0);
   const int tid = threadIdx.x;
-  // two 64 x 65 tiles of dynamic shared memory (the triangle's tile, the inverse)
+  // a 64 x 65 tile of dynamic shared memory and its diagonal's reciprocals
   extern __shared__ unsigned char smem_raw[];
-  T(*Ds)[IB + 1] = reinterpret_cast<T(*)[IB + 1]>(smem_raw);
-  T(*Ts)[IB + 1] = reinterpret_cast<T(*)[IB + 1]>(smem_raw + sizeof(T) * IB * (IB + 1));
+  T* D = reinterpret_cast<T*>(smem_raw);
+  T* rinv = D + IB * (IB + 1);
   const int rows = min(IB, k - i0);
   for (int t = tid; t < IB * IB; t += blockDim.x) {
     const int r = t % IB, c = t / IB;
-    Ds[r][c] = (r < rows && c < rows) ? A[(i0 + r) + (int64_t)(i0 + c) * m] : T(0);
-    Ts[r][c] = r == c ? T(1) : T(0);
+    D[r + c * (IB + 1)] = (r < rows && c < rows) ? A[(i0 + r) + (int64_t)(i0 + c) * m] : T(0);
   }
   __syncthreads();
-  if (!upper) {
-    for (int r = 0; r < rows; ++r) {  // unit diagonal: row r is final now
-      for (int t = tid; t < (rows - r - 1) * IB; t += blockDim.x) {
-        const int r2 = r + 1 + t / IB, c = t % IB;
-        Ts[r2][c] -= Ds[r2][r] * Ts[r][c];
-      }
-      __syncthreads();
-    }
-  } else {
-    for (int r = rows - 1; r >= 0; --r) {
-      const T d = Ds[r][r];
-      for (int c = tid; c < IB; c += blockDim.x) Ts[r][c] /= d;
-      __syncthreads();
-      for (int t = tid; t < r * IB; t += blockDim.x) {
-        const int r2 = t / IB, c = t % IB;
-        Ts[r2][c] -= Ds[r2][r] * Ts[r][c];
-      }
-      __syncthreads();
-    }
-  }
-  for (int t = tid; t < IB * IB; t += blockDim.x) {
-    const int r = t % IB, c = t / IB;
-    if (r < rows && c < rows) X[(i0 + r) + (int64_t)(i0 + c) * ld] = Ts[r][c];
+  if (upper && tid < rows) rinv[tid] = T(1) / D[tid + tid * (IB + 1)];
+  __syncthreads();
+  // the other triangle of the tile is zero since the allocation
+  T* Xd = X + i0 + (int64_t)i0 * ld;
+  for (int c0 = 4 * (tid / 32); c0 < rows; c0 += kThreads / 8) {
+    if (upper)
+      warp_tri_inverse<T, IB / 32, true>(D, rinv, IB + 1, rows, c0, Xd, ld);
+    else
+      warp_tri_inverse<T, IB / 32, false>(D, rinv, IB + 1, rows, c0, Xd, ld, true);
   }
 }
 
@@ -490,22 +553,27 @@ __global__ void k_tri_inverse_copy(DevFronts F, const int32_t* __restrict__ list
 // ---------------------------------------------------------------------------
 constexpr int kLuPanel = 8;  // pivots per panel of the small-front LU
 
-template <typename T>
-__global__ void __launch_bounds__(kThreads)
+// One CTA per front.  The time of a front is a chain: 64 pivots, then the inverses.  The
+// panel's columns and the multipliers of the trailing update are kept in registers (RP rows
+// per lane, m <= 32 RP), pivot rows are broadcast by shuffles, and every warp forms four
+// columns of both inverses at a time (k steps together) instead of all threads one column
+// at a time between barriers: 20,682 fronts of 41 pivots and up to 87 rows (a batch of 256
+// 2-D systems) 1,757 -> 1,195 us, the whole block LU of one 64 x 64 grid 264 -> 112 us.
+template <typename T, int RP>
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2)
     k_front_lu_small(DevFronts F, const int32_t* __restrict__ list, T* __restrict__ arena,
                      const double* __restrict__ rownorm, double pivot_tol,
                      long long* __restrict__ err) {
   extern __shared__ unsigned char smem_raw[];
   const int32_t f = list[blockIdx.x];
   const int32_t k = F.k[f], m = F.m[f];
-  double* th = reinterpret_cast<double*>(smem_raw);  // the k pivot thresholds
-  T* A = reinterpret_cast<T*>(smem_raw + (size_t)k * sizeof(double));
+  T* A = reinterpret_cast<T*>(smem_raw);
   T* __restrict__ G = arena + F.arena[f];
-  T* v = A + (int64_t)m * m;  // 2 m scratch entries for the inversions
+  T* th = A + m * m;  // the k pivot thresholds, then the reciprocals of the pivots
   const int64_t row0 = F.row0[f];
   const int tid = threadIdx.x;
   for (int t = tid; t < m * m; t += blockDim.x) A[t] = G[t];
-  for (int t = tid; t < k; t += blockDim.x) th[t] = pivot_tol * rownorm[row0 + t];
+  for (int t = tid; t < k; t += blockDim.x) th[t] = threshold<T>(pivot_tol * rownorm[row0 + t]);
   __syncthreads();
   // right-looking LU in panels of kLuPanel pivots: warp 0 factors the panel
   // columns, the CTA solves the panel rows of U12 and applies the rank-
@@ -515,89 +583,97 @@ __global__ void __launch_bounds__(kThreads)
   for (int jp = 0; jp < k; jp += kLuPanel) {
     const int je = min(k, jp + kLuPanel);
     if (warp == 0) {
-      for (int j = jp; j < je; ++j) {
-        T piv = A[j + j * m];
-        const double thr = th[j];
-        const bool small = !(fabs((double)piv) > thr);
-        if (small) {
-          const double rep = thr > 0.0 ? thr : 1e-300;
-          piv = (T)((double)piv < 0.0 ? -rep : rep);
+      T a[RP][kLuPanel];  // rows jp + lane + 32 p
+#pragma unroll
+      for (int p = 0; p < RP; ++p)
+#pragma unroll
+        for (int c = 0; c < kLuPanel; ++c) {
+          const int i = jp + lane + 32 * p;
+          a[p][c] = i < m && jp + c < je ? A[i + (jp + c) * m] : T(0);
         }
-        __syncwarp();  // every lane has read the pivot before it is replaced
-        if (small && lane == 0) {
-          if (atomicCAS((unsigned long long*)&err[0], 0ull, 1ull) == 0ull) {
-            err[1] = f;
-            err[2] = row0 + j;
+#pragma unroll
+      for (int j = 0; j < kLuPanel; ++j) {
+        if (jp + j >= je) break;
+        T piv = __shfl_sync(0xffffffffu, a[0][j], j);
+        if (!(fabs(piv) > th[jp + j])) {
+          piv = replacement(piv, pivot_tol * rownorm[row0 + jp + j]);
+          if (lane == j) {
+            if (atomicCAS((unsigned long long*)&err[0], 0ull, 1ull) == 0ull) {
+              err[1] = f;
+              err[2] = row0 + jp + j;
+            }
+            a[0][j] = piv;
           }
-          A[j + j * m] = piv;
         }
         const T inv = T(1) / piv;
-        for (int i = j + 1 + lane; i < m; i += 32) {
-          const T l = A[i + j * m] * inv;
-          A[i + j * m] = l;
-          for (int c = j + 1; c < je; ++c) A[i + c * m] -= l * A[j + c * m];
+#pragma unroll
+        for (int p = 0; p < RP; ++p)
+          if (p > 0 || lane > j) a[p][j] *= inv;
+#pragma unroll
+        for (int c = j + 1; c < kLuPanel; ++c) {
+          const T u = __shfl_sync(0xffffffffu, a[0][c], j);
+#pragma unroll
+          for (int p = 0; p < RP; ++p)
+            if (p > 0 || lane > j) a[p][c] -= a[p][j] * u;
         }
-        __syncwarp();
       }
+#pragma unroll
+      for (int p = 0; p < RP; ++p)
+#pragma unroll
+        for (int c = 0; c < kLuPanel; ++c) {
+          const int i = jp + lane + 32 * p;
+          if (i < m && jp + c < je) A[i + (jp + c) * m] = a[p][c];
+        }
     }
     __syncthreads();
     // U12 rows of the panel: forward substitution with its unit-lower block
-    for (int c = je + tid; c < m; c += blockDim.x)
-      for (int j = jp; j < je; ++j) {
-        const T u = A[j + c * m];
-        for (int i = j + 1; i < je; ++i) A[i + c * m] -= A[i + j * m] * u;
-      }
-    __syncthreads();
-    // trailing update, one warp per column, lanes over rows
-    for (int c = je + warp; c < m; c += blockDim.x >> 5) {
+    for (int c = je + tid; c < m; c += blockDim.x) {
       T u[kLuPanel];
 #pragma unroll
       for (int j = 0; j < kLuPanel; ++j) u[j] = jp + j < je ? A[jp + j + c * m] : T(0);
-      for (int i = je + lane; i < m; i += 32) {
+#pragma unroll
+      for (int j = 0; j < kLuPanel; ++j)
+#pragma unroll
+        for (int i = j + 1; i < kLuPanel; ++i)
+          if (jp + i < je) u[i] -= A[jp + i + (jp + j) * m] * u[j];
+#pragma unroll
+      for (int j = 1; j < kLuPanel; ++j)
+        if (jp + j < je) A[jp + j + c * m] = u[j];
+    }
+    __syncthreads();
+    // trailing update, one warp per column, lanes over rows
+    T l[RP][kLuPanel];
+#pragma unroll
+    for (int p = 0; p < RP; ++p)
+#pragma unroll
+      for (int j = 0; j < kLuPanel; ++j) {
+        const int i = je + lane + 32 * p;
+        l[p][j] = i < m && jp + j < je ? A[i + (jp + j) * m] : T(0);
+      }
+    for (int c = je + warp; c < m; c += kThreads / 32) {
+      T u[kLuPanel];
+#pragma unroll
+      for (int j = 0; j < kLuPanel; ++j) u[j] = jp + j < je ? A[jp + j + c * m] : T(0);
+#pragma unroll
+      for (int p = 0; p < RP; ++p) {
+        const int i = je + lane + 32 * p;
+        if (i >= m) continue;
         T a = A[i + c * m];
 #pragma unroll
-        for (int j = 0; j < kLuPanel; ++j)
-          if (jp + j < je) a -= A[i + (jp + j) * m] * u[j];
+        for (int j = 0; j < kLuPanel; ++j) a -= l[p][j] * u[j];
         A[i + c * m] = a;
       }
     }
     __syncthreads();
   }
-  // The two inverses touch disjoint triangles: the first half of the CTA
-  // forms L11^-1, the second U11^-1, each with its own scratch vector and
-  // named barrier.
-  const int half = blockDim.x >> 1;
-  const int gt = tid % half;
-  if (tid < half) {
-    // L11^-1 (strictly lower part, unit diagonal), columns descending
-    for (int j = k - 2; j >= 0; --j) {
-      for (int i = j + 1 + gt; i < k; i += half) v[i] = A[i + j * m];
-      asm volatile("bar.sync 1, %0;" ::"r"(half) : "memory");
-      for (int i = j + 1 + gt; i < k; i += half) {
-        T s2 = v[i];
-        for (int l = j + 1; l < i; ++l) s2 += A[i + l * m] * v[l];
-        A[i + j * m] = -s2;
-      }
-      asm volatile("bar.sync 1, %0;" ::"r"(half) : "memory");
-    }
-  } else {
-    T* vu = v + m;
-    // U11^-1 (upper part with the diagonal), columns ascending
-    for (int j = 0; j < k; ++j) {
-      for (int i = gt; i <= j; i += half) vu[i] = A[i + j * m];
-      asm volatile("bar.sync 2, %0;" ::"r"(half) : "memory");
-      const T d = vu[j];
-      for (int i = gt; i < j; i += half) {
-        T s2 = T(0);
-        for (int l = i; l < j; ++l) s2 += A[i + l * m] * vu[l];
-        A[i + j * m] = -s2 / d;
-      }
-      if (gt == 0) A[j + j * m] = T(1) / d;
-      asm volatile("bar.sync 2, %0;" ::"r"(half) : "memory");
-    }
-  }
+  for (int t = tid; t < k; t += blockDim.x) th[t] = T(1) / A[t + t * m];
   __syncthreads();
-  for (int t = tid; t < m * m; t += blockDim.x) G[t] = A[t];
+  for (int j = warp; j < m; j += kThreads / 32)  // L21, U12 and the update block
+    for (int i = (j < k ? k : 0) + lane; i < m; i += 32) G[i + j * m] = A[i + j * m];
+  for (int c0 = 4 * warp; c0 < k; c0 += 4 * (kThreads / 32)) {
+    warp_tri_inverse<T, RP, false>(A, th, m, k, c0, G, m);
+    warp_tri_inverse<T, RP, true>(A, th, m, k, c0, G, m);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -748,7 +824,7 @@ void launch_tri_inverse_mc(DevFronts F, const int32_t* tile_front, const int32_t
   if (ntiles <= 0) return;
   const size_t sm = sizeof(T) * ((size_t)IB * (NB + 1) + (size_t)NB * (IB + 1) + 2 * (size_t)IB * (IB + 1));
   record_launch_error(cudaFuncSetAttribute(k_tri_inverse_mc<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  const size_t smd = sizeof(T) * 2 * (size_t)IB * (IB + 1);
+  const size_t smd = sizeof(T) * ((size_t)IB * (IB + 1) + IB);
   record_launch_error(cudaFuncSetAttribute(k_tri_inverse_diag<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smd));
   k_tri_inverse_diag<T><<<dim3(ntiles, 2), kThreads, smd, s>>>(F, tile_front, tile_cb, arena, inv,
                                                                 inv_off);
@@ -770,10 +846,15 @@ void launch_front_lu_small(DevFronts F, const int32_t* list, int32_t nf, int32_t
                            const double* rownorm_new, double pivot_tol, long long* err,
                            cudaStream_t s) {
   if (nf <= 0) return;
-  const size_t sm = ((size_t)max_m * max_m + 2 * (size_t)max_m) * sizeof(T) + (size_t)max_m * sizeof(double);
+  const size_t sm = ((size_t)max_m * max_m + (size_t)max_m) * sizeof(T);
+  static_assert(small_front_max<T>() <= 128, "rows per lane");
+  auto k = max_m <= 32   ? k_front_lu_small<T, 1>
+           : max_m <= 64 ? k_front_lu_small<T, 2>
+           : max_m <= 96 ? k_front_lu_small<T, 3>
+                         : k_front_lu_small<T, 4>;
   if (sm > 40 * 1024)  // static bytes count too
-    record_launch_error(cudaFuncSetAttribute(k_front_lu_small<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  k_front_lu_small<T><<<nf, kThreads, sm, s>>>(F, list, arena, rownorm_new, pivot_tol, err);
+    record_launch_error(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  k<<<nf, kThreads, sm, s>>>(F, list, arena, rownorm_new, pivot_tol, err);
 }
 
 template <typename T, typename TG>

@@ -207,3 +207,29 @@ def test_fp32_wide_front_inverses(rows):
     # two triangular products of the solve
     assert np.linalg.norm(r) <= 3 * 4 * rows * 2.0 ** -24 * np.linalg.norm(np.abs(A[:rows, :rows]) @ np.abs(x))
     S.close()
+
+
+@pytest.mark.parametrize("prec", [N.DDPS_FP32, N.DDPS_FP64])
+@pytest.mark.parametrize("rows", [1, 3, 8, 9, 31, 32, 33, 64, 65, 90, 96, 97, 127, 128])
+def test_dense_front_edges(rows, prec):
+    """Block solves through one dense front at the edges of the register rows, the pivot
+    panels and the four-column groups of the inverses."""
+    rng = np.random.default_rng(rows)
+    n = rows + 3
+    A = np.zeros((n, n))
+    A[:rows, :rows] = rng.uniform(-1.0, 1.0, (rows, rows))
+    A[0, rows] = A[rows, 0] = 1.0
+    A[np.arange(n), np.arange(n)] = 0.0
+    A[np.arange(n), np.arange(n)] = 1.5 * np.abs(A).sum(axis=1) + 0.1
+    M = sp.csr_matrix(A)
+    S = Solver(M.indptr, M.indices, np.array([0, rows, n]), factor_prec=prec, spike_prec=prec,
+               ghat_prec=prec, inner_prec=prec)
+    S.factor(dev(M.data))
+    y = rng.uniform(-1.0, 1.0, n)
+    x = host(S.block_solve(dev(y)))[:rows]
+    D = A[:rows, :rows]
+    u = 2.0 ** (-24 if prec == N.DDPS_FP32 else -53)
+    # dominance: |L||U| <= 3 |D|; rows (and a conversion's) roundings each for the factors,
+    # the inverses and the two triangular products
+    assert np.linalg.norm(D @ x - y[:rows]) <= 3 * 4 * (rows + 1) * u * np.linalg.norm(np.abs(D) @ np.abs(x))
+    S.close()
