@@ -1237,9 +1237,11 @@ double inner_solve(ddps_handle* h, const double* ghat64, double* zhat64, const d
   CK(cudaMemcpyAsync(rh, r, m * sizeof(TI), cudaMemcpyDeviceToDevice, s));
   // Iterations are enqueued without waiting: the convergence tests run on the
   // device (fused into the reductions), stopped systems skip every kernel, and
-  // the host looks at a single "some system still iterating" flag every
-  // kCheckEvery iterations.
-  constexpr int kCheckEvery = 4;
+  // the host looks at a single "some system still iterating" flag every four
+  // iterations; after each one when the products are implicit, as these are not skipped
+  // (64^3: an iteration takes 560 us, a look 20; the step 33.5 -> 31.1 ms).  A loop node that
+  // decides on the device costs as much per pass as the looks it saves.
+  const int check_every = h->opt.ghat_mode == DDPS_GHAT_IMPLICIT ? 1 : 4;
   const bool graphed = graphs_on(h) && h->opt.maxit_in > 0;
   // rho and beta of the first iteration; every later iteration's come from
   // the previous one's update of r (POST_CHECK_FULL_BETA)
@@ -1292,21 +1294,21 @@ double inner_solve(ddps_handle* h, const double* ghat64, double* zhat64, const d
     h->launches += 3;  // the two G^ products count their own launches
   };
   if (graphed) {
-    // kCheckEvery iterations and the "some system still iterating" flag, one
+    // check_every iterations and the "some system still iterating" flag, one
     // graph replayed until every system has stopped (the device counter
     // stops a system after maxit_in iterations)
     if (!h->g_inner)
       h->g_inner = capture_graph(
           h,
           [&](cudaStream_t gs) {
-            for (int q = 0; q < kCheckEvery; ++q) iteration(-h->opt.maxit_in, gs);
+            for (int q = 0; q < check_every; ++q) iteration(-h->opt.maxit_in, gs);
             any_active(ns, sc, h->any_flag, gs);
             CK(cudaMemcpyAsync(h->any_host, h->any_flag, sizeof(int32_t), cudaMemcpyDeviceToHost,
                                gs));
             h->launches++;
           },
           &h->g_inner_launches);
-    for (int it = 0; it < h->opt.maxit_in; it += kCheckEvery) {
+    for (int it = 0; it < h->opt.maxit_in; it += check_every) {
       replay_graph(h, h->g_inner, h->g_inner_launches, s);
       CK(cudaStreamSynchronize(s));
       h->stage_next = 0;
@@ -1314,7 +1316,7 @@ double inner_solve(ddps_handle* h, const double* ghat64, double* zhat64, const d
     }
   } else {
     for (int it = 1; it <= h->opt.maxit_in; ++it) {
-      if ((it - 1) % kCheckEvery == 0) {
+      if ((it - 1) % check_every == 0) {
         any_active(ns, sc, h->any_flag, s);
         CK(cudaMemcpyAsync(h->any_host, h->any_flag, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
