@@ -93,8 +93,8 @@ struct Vec<__nv_bfloat16> {
 // pairs of floats (hi + lo, about 48 bits; products by fused multiply-add, sums by
 // Knuth's two-sum), because the FP64 pipe runs a warp instruction in 64 cycles here:
 // with FP64 sums, scalars and updates an iteration of a 384-row system took 18 us,
-// with pairs 4.  Pairs have FP32's range, so the system is scaled by the power of
-// two that brings ||g|| to [1, 2).
+// with pairs 12 (and 7.8 with fewer barriers, too).  Pairs have FP32's range, so the
+// system is scaled by the power of two that brings ||g|| to [1, 2).
 struct Pair {
   float hi, lo;
 };

@@ -768,13 +768,19 @@ __device__ __forceinline__ void fused_dims(int32_t k, int32_t m, int& nout, int&
 // factored front are copied, the product blocks are formed here in fp32:
 //   backward, column j >= k:  -sum_{l >= i} U11^-1(i, l) U12(l, j)
 //   forward,  row i >= k:     -sum_{l >= j} L21(i, l) L11^-1(l, j)
-// The right factor's 32 columns are staged in shared memory ([k][33]).
+// The right factor's 32 columns are staged in shared memory.  A thread forms 8 columns of a
+// row (lanes on consecutive rows: coalesced reads of the left factor, broadcast 16-byte reads
+// of the right one, 16-byte stores): a row's chain of k steps is 8 multiply-adds wide, where a
+// thread per row (forward, most threads idle for small fronts) and a warp per row (backward)
+// took 32 and one load per step.  A batch of 256 2-D
+// systems: forward 1,326 -> 763 us, backward 1,015 -> 790; 300k band: backward 6.1 -> 2.1 ms.
+constexpr int WP_LD = TC_BK + 4;  // row stride of the staged factor (16-byte aligned)
 template <int DIR, int PASSES>
 __global__ void __launch_bounds__(TC_THREADS)
     k_w_pack(DevFronts F, const int32_t* __restrict__ fronts, const int32_t* __restrict__ kbs,
              const int64_t* __restrict__ woff, const float* __restrict__ arena,
              unsigned char* __restrict__ wpk) {
-  extern __shared__ float Rs[];
+  extern __shared__ __align__(16) float Rs[];
   const int32_t f = fronts[blockIdx.x];
   const int32_t k = F.k[f], m = F.m[f];
   int nout, K;
@@ -785,80 +791,77 @@ __global__ void __launch_bounds__(TC_THREADS)
   const float* __restrict__ A = arena + F.arena[f];
   const int j0 = kb * TC_BK;
   // right factor: backward U12(l, j) (rows l < k of column j >= k), forward L11^-1(l, j)
-  for (int e = threadIdx.x; e < k * TC_BK; e += TC_THREADS) {
-    const int l = e % k, jj = e / k, j = j0 + jj;
-    float v = 0.f;
-    if (j < K) {
-      if (DIR == DIR_BWD)
-        v = j >= k ? A[l + (int64_t)j * m] : 0.f;
-      else
-        v = l > j ? A[l + (int64_t)j * m] : (l == j ? 1.f : 0.f);
+  for (int jj = threadIdx.x / 32; jj < TC_BK; jj += TC_THREADS / 32) {
+    const int j = j0 + jj;
+    for (int l = threadIdx.x % 32; l < k; l += 32) {
+      float v = 0.f;
+      if (j < K) {
+        if (DIR == DIR_BWD)
+          v = j >= k ? A[l + (int64_t)j * m] : 0.f;
+        else
+          v = l > j ? A[l + (int64_t)j * m] : (l == j ? 1.f : 0.f);
+      }
+      Rs[l * WP_LD + jj] = v;
     }
-    Rs[l * (TC_BK + 1) + jj] = v;
   }
   __syncthreads();
   const uint32_t part = (uint32_t)nf * TC_BK * 2;
   unsigned char* dst = wpk + woff[f] + (int64_t)kb * (PASSES == 3 ? 2 : 1) * part;
-  if constexpr (DIR == DIR_FWD) {
-  // forward (m output rows): one thread per row, the 32 entries of the row in
-  // this K-block as outer products (a coalesced column read of L21 per term,
-  // the row of L11^-1 from shared memory), then 16-byte stores
-  for (int i = threadIdx.x; i < nf; i += TC_THREADS) {
-    float acc[TC_BK];
+  constexpr int kRows = TC_THREADS / (TC_BK / 8);
+  const int kc = threadIdx.x / kRows;  // this thread's 8 columns
+  const int jc = j0 + kc * 8;
+  for (int i = threadIdx.x % kRows; i < nf; i += kRows) {
+    float v[8];
 #pragma unroll
-    for (int jj = 0; jj < TC_BK; ++jj) acc[jj] = 0.f;
-    if (i < nout && i >= k) {
-      for (int l = j0; l < k; ++l) {  // -sum_l L21(i, l) L11^-1(l, j); L11^-1(l, j) = 0 for l < j
-        const float a = A[i + (int64_t)l * m];
-        const float* __restrict__ r = Rs + l * (TC_BK + 1);
+    for (int t = 0; t < 8; ++t) v[t] = 0.f;
+    // rows with a product: forward the update rows, backward every row if columns j >= k are here
+    const bool prod = DIR == DIR_FWD ? i < nout && i >= k : i < nout && jc + 7 >= k;
+    if (prod) {
+      constexpr int NA = DIR == DIR_BWD ? 2 : 1;  // partial sums
+      float acc[NA][8];
 #pragma unroll
-        for (int jj = 0; jj < TC_BK; ++jj) acc[jj] = fmaf(a, r[jj], acc[jj]);
+      for (int q = 0; q < NA; ++q)
+#pragma unroll
+        for (int t = 0; t < 8; ++t) acc[q][t] = 0.f;
+      // L11^-1(l, j) = 0 for l < j, U11^-1(i, l) = 0 for l < i
+      int l = DIR == DIR_FWD ? j0 : (i & ~31);
+      auto term = [&](int q, int ll, float a) {
+        const float4 x = *reinterpret_cast<const float4*>(Rs + ll * WP_LD + kc * 8);
+        const float4 y = *reinterpret_cast<const float4*>(Rs + ll * WP_LD + kc * 8 + 4);
+        acc[q][0] = fmaf(a, x.x, acc[q][0]);
+        acc[q][1] = fmaf(a, x.y, acc[q][1]);
+        acc[q][2] = fmaf(a, x.z, acc[q][2]);
+        acc[q][3] = fmaf(a, x.w, acc[q][3]);
+        acc[q][4] = fmaf(a, y.x, acc[q][4]);
+        acc[q][5] = fmaf(a, y.y, acc[q][5]);
+        acc[q][6] = fmaf(a, y.z, acc[q][6]);
+        acc[q][7] = fmaf(a, y.w, acc[q][7]);
+      };
+      constexpr int NL = DIR == DIR_FWD ? 8 : 4;  // loads of the left factor in flight
+      for (; l + NL <= k; l += NL) {
+        float a[NL];
+#pragma unroll
+        for (int q = 0; q < NL; ++q) a[q] = DIR == DIR_FWD || l + q >= i ? A[i + (int64_t)(l + q) * m] : 0.f;
+#pragma unroll
+        for (int q = 0; q < NL; ++q) term(q % NA, l + q, a[q]);
       }
-    }
+      for (; l < k; ++l) term(0, l, DIR == DIR_FWD || l >= i ? A[i + (int64_t)l * m] : 0.f);
 #pragma unroll
-    for (int kc = 0; kc < TC_BK / 8; ++kc) {
-      float v[8];
+      for (int t = 0; t < 8; ++t) v[t] = NA == 2 ? -(acc[0][t] + acc[NA - 1][t]) : -acc[0][t];
+    }
+    // entries that are blocks of the factored front
 #pragma unroll
-      for (int t = 0; t < 8; ++t) {
-        const int jj = kc * 8 + t, j = j0 + jj;
-        float w = 0.f;
-        if (i < nout && j < K)
-          w = i < k ? (i > j ? A[i + (int64_t)j * m] : (i == j ? 1.f : 0.f)) : -acc[jj];
-        v[t] = w;
-      }
-      const uint32_t off = chunk_off(i, kc);
-      store_split(dst + off, dst + part + off, v, PASSES == 3);
+    for (int t = 0; t < 8; ++t) {
+      const int j = jc + t;
+      if (i >= nout || j >= K)
+        v[t] = 0.f;
+      else if (DIR == DIR_FWD && i < k)
+        v[t] = i > j ? A[i + (int64_t)j * m] : (i == j ? 1.f : 0.f);
+      else if (DIR == DIR_BWD && j < k)
+        v[t] = i <= j ? A[i + (int64_t)j * m] : 0.f;
     }
-  }
-  } else {
-  // backward (k output rows, often few): one warp per row, lanes over the
-  // 32 columns; -sum_{l >= i} U11^-1(i, l) U12(l, j) for the columns j >= k
-  const int jj = threadIdx.x & 31;
-  const int j = j0 + jj;
-  for (int i = threadIdx.x >> 5; i < nf; i += TC_THREADS / 32) {
-    float w = 0.f;
-    if (i < nout && j < K) {
-      if (j < k) {
-        w = i <= j ? A[i + (int64_t)j * m] : 0.f;
-      } else {
-        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-        int l = i;
-        for (; l + 4 <= k; l += 4) {
-          a0 = fmaf(A[i + (int64_t)l * m], Rs[l * (TC_BK + 1) + jj], a0);
-          a1 = fmaf(A[i + (int64_t)(l + 1) * m], Rs[(l + 1) * (TC_BK + 1) + jj], a1);
-          a2 = fmaf(A[i + (int64_t)(l + 2) * m], Rs[(l + 2) * (TC_BK + 1) + jj], a2);
-          a3 = fmaf(A[i + (int64_t)(l + 3) * m], Rs[(l + 3) * (TC_BK + 1) + jj], a3);
-        }
-        for (; l < k; ++l) a0 = fmaf(A[i + (int64_t)l * m], Rs[l * (TC_BK + 1) + jj], a0);
-        w = -((a0 + a1) + (a2 + a3));
-      }
-    }
-    uint16_t hi, lo;
-    split_bf16(w, hi, lo);
-    const uint32_t off = chunk_off(i, jj >> 3) + (jj & 7) * 2;
-    *reinterpret_cast<uint16_t*>(dst + off) = hi;
-    if (PASSES == 3) *reinterpret_cast<uint16_t*>(dst + part + off) = lo;
-  }
+    const uint32_t off = chunk_off(i, kc);
+    store_split(dst + off, dst + part + off, v, PASSES == 3);
   }
 }
 
@@ -1557,7 +1560,7 @@ void launch_tc_w_pack(int bwd, int passes, DevFronts F, const int32_t* fronts, c
                       int32_t nitems, int32_t max_k, const int64_t* woff, const float* arena,
                       unsigned char* wpk, cudaStream_t s) {
   if (nitems <= 0) return;
-  const size_t sm = (size_t)std::max(max_k, 1) * (TC_BK + 1) * sizeof(float);
+  const size_t sm = (size_t)std::max(max_k, 1) * WP_LD * sizeof(float);
 #define DDPS_WPACK(D, P)                                                                        \
   record_launch_error(cudaFuncSetAttribute(k_w_pack<D, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));   \
   k_w_pack<D, P><<<nitems, TC_THREADS, sm, s>>>(F, fronts, kb, woff, arena, wpk);
