@@ -1954,15 +1954,18 @@ void pack_ilu(ddps_handle* h, int64_t fs) {
 }
 
 // Whether the FP64 spike products run in fixed point on the tensor cores: always the faster
-// (24^2, three blocks: 0.49 -> 0.45 ms a factorisation; 48^3, eight slabs: 278 -> 64), but the
-// digits take 14 bytes per entry of the factors, and past 24 GB those stay with the panels.
+// (24^2, three blocks: 0.49 -> 0.45 ms a factorisation; 48^3, eight slabs: 278 -> 62), but the
+// digits take 14 bytes per entry of the factors: not past 24 GB, nor where what is left of the
+// device's memory (factors, G^ and panels are allocated) would not hold them and the vectors.
 bool oz_wins(const Analysis& A) {
   int64_t bytes = 0;
   for (size_t f = 0; f < A.f_k.size(); ++f) {
     const int32_t k = A.f_k[f], r = A.f_m[f] - k, tk = (k + oz_tile_m() - 1) / oz_tile_m(), tr = (r + oz_tile_m() - 1) / oz_tile_m();
     bytes += tk * (2 * oz_tile_bytes(k) + oz_tile_bytes(r)) + tr * oz_tile_bytes(k);
   }
-  return bytes <= (int64_t)24 << 30;
+  size_t left = 0, total = 0;
+  CK(cudaMemGetInfo(&left, &total));
+  return bytes <= (int64_t)24 << 30 && bytes + 40 * 8 * A.n + ((int64_t)1 << 30) <= (int64_t)left;
 }
 
 // Triangular inverses of the wide FP32 fronts from those of their diagonal blocks, two

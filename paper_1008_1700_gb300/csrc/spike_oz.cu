@@ -14,16 +14,16 @@
 // long-double solution: 1.8e-16 .. 2.8e-16 relative (2.5e-16 .. 3.7e-16 with FP64 FMAs).
 //
 // The products are bound by latency and issue slots, not by the MMAs (13% of the tensor
-// pipe at the roots, 3 to 8% below): cutting an entry costs some 50 instructions, rounding a
+// pipe at the roots, 3 to 8% below them): cutting an entry costs some 50 instructions, rounding a
 // result 80, and most fronts have one to four 32-column stages.  So a CTA of 512 threads takes
 // 32 front rows (N of the MMA) times 128 panel columns (M: a thread holds a column, its
 // accesses are coalesced), with 64 registers and 256 tensor-memory columns, and two CTAs
 // share an SM: one's loads and rounding run beside the other's products.  A's digits are cut
 // once per factorisation (k_oz_pack) and come with one bulk copy per stage; B's are cut by
 // all threads from the panel, in integer arithmetic.  48^3, eight slabs, FP64: forward and
-// backward products 54.7 + 207 -> 12.5 + 36.2 ms, the packing (0.9 ms) included; tiles of 64
-// rows, one CTA per SM: 12.7 + 40.7 ms with 1,024 threads, 14.2 + 45.2 with 512; 128 rows by
-// 64 columns: 18.9 + 67.4.
+// backward products 54.7 + 207 -> 12.0 + 34.7 ms, the packing (0.9 ms) included (the zero
+// halves of the triangles skipped; 12.5 + 36.2 with them); tiles of 64 rows, one CTA per SM:
+// 12.7 + 40.7 ms with 1,024 threads, 14.2 + 45.2 with 512; 128 rows by 64 columns: 18.9 + 67.4.
 // Every wait is bounded; a wait that runs out records error code 2.
 #include <cuda_runtime.h>
 
