@@ -437,10 +437,25 @@ struct Work {
 
 int64_t up4(int64_t n) { return (n + 3) / 4 * 4; }
 
+// Floats of the split sums of any batch up to B: a batch one above a multiple of 64 takes fewer
+// splits and so less than the one before it, but a buffer for the full batch also has to hold
+// the ragged last one.
+int64_t split_floats(int32_t hidden, int32_t d_out, int32_t B) {
+  const int K = d_out > hidden ? d_out : hidden;
+  int64_t most = up4((int64_t)B * hidden);
+  for (int64_t b = BM;; b += BM) {
+    const int32_t rows = (int32_t)(b < B ? b : B);
+    const int ns = split_count(rows, hidden, K);
+    const int64_t n = ns * up4((int64_t)rows * hidden);
+    if (n > most) most = n;
+    if (rows == B || ns == 1) return most;
+  }
+}
+
 int64_t work_bytes(int32_t hidden, int32_t layers, int32_t d_out, int32_t B) {
   const int64_t hb = up4((int64_t)B * hidden);
-  const int ns = split_count(B, hidden, d_out > hidden ? d_out : hidden);
-  return 4 * ((layers + 2 + ns) * hb + up4((int64_t)B * d_out)) + 8 * (int64_t)loss_blocks(B, d_out) + 256;
+  return 4 * ((layers + 2) * hb + split_floats(hidden, d_out, B) + up4((int64_t)B * d_out)) +
+         8 * (int64_t)loss_blocks(B, d_out) + 256;
 }
 
 Work carve(void* ws, int32_t hidden, int32_t layers, int32_t d_out, int32_t B) {
@@ -458,7 +473,7 @@ Work carve(void* ws, int32_t hidden, int32_t layers, int32_t d_out, int32_t B) {
   w.dA1 = p;
   p += hb;
   w.split = p;
-  p += split_count(B, hidden, d_out > hidden ? d_out : hidden) * hb;
+  p += split_floats(hidden, d_out, B);
   w.partial = (double*)p;
   return w;
 }

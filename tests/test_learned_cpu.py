@@ -7,6 +7,7 @@ import numpy as np
 import pytest
 import torch
 
+from paper_1008_1700_gb300 import native as N
 from paper_1008_1700_gb300.learned import GuessNet, StepGuess
 
 
@@ -68,3 +69,10 @@ def test_checkpoints_of_another_kind_or_shape_are_rejected(tmp_path):
         np.savez(f, params=arrays["params"])
     with pytest.raises(ValueError, match="no checkpoint metadata"):
         GuessNet.load(p_none, device="cpu")
+
+
+@pytest.mark.parametrize("hidden,layers,d_out", [(256, 3, 32256), (256, 3, 1000), (31, 1, 7), (512, 2, 9000)])
+def test_workspace_grows_with_the_batch(hidden, layers, d_out):
+    """A workspace sized for the full batch holds every smaller one, the ragged last one too."""
+    sizes = [N.ddps_mlp_workspace_bytes(2, hidden, layers, d_out, B) for B in range(1, 700)]
+    assert all(a <= b for a, b in zip(sizes, sizes[1:]))
