@@ -96,9 +96,8 @@ typedef struct {
   int32_t factor_prec;    /* FP64 or FP32: storage and arithmetic of the block factors (Fig. 2 step 2)
                              and of the block solves 6.1 / 6.5 */
   int32_t spike_prec;     /* operands of the spike products of Fig. 2 step 4: equal to factor_prec
-                             (FP64: exact sums of 55-bit fixed-point operands, rounded once;
-                             FP32: SIMT), or, with FP32 factors, BF16 / BF16X3 (tensor cores,
-                             fp32 accumulation) */
+                             (FMAs), or, with FP32 factors, BF16 / BF16X3 (tensor cores, fp32
+                             accumulation) */
   int32_t ghat_prec;      /* FP64, FP32, FP16 or BF16 storage of G^ (Sec. 3: dense per-partition
                              arrays); FP16/BF16 products accumulate in FP32 */
   int32_t inner_prec;     /* FP64 or FP32 vectors of the inner BiCGStab on G^ (6.3) */

@@ -234,9 +234,6 @@ struct ddps_handle : SolveWork {
   std::vector<int64_t> fz_ptr;
   int32_t tc_max_kt[4] = {0, 0, 0, 0};
   int tc_passes = 0;
-  bool oz = false;  // FP64 spikes: fixed-point products, digits of A packed in atc
-  OzUnits oz_u{};
-  int32_t* oz_work = nullptr;
   double *im_q = nullptr, *im_g = nullptr;  // implicit G^: R~ v and D~^-1 R~ v
   // host-buffer entry points stage f and x here
   double *io_f = nullptr, *io_x = nullptr;
@@ -508,13 +505,6 @@ void spike_op(ddps_handle* h, int op, const int32_t* tf, const int32_t* tm, cons
       return;
     }
   }
-  if constexpr (std::is_same<T, double>::value) {
-    if (h->oz) {
-      launch_spike_gemm_oz(op, h->F, h->oz_u, tf, tm, ta, h->atc, nt, h->block_ncols, j0, h->NR, X, Tb,
-                           h->derr, s);
-      return;
-    }
-  }
   launch_spike_gemm<T>(op, h->F, tf, tm, nt, arena, h->block_ncols, j0, h->NR, X, Tb, s);
 }
 
@@ -683,22 +673,6 @@ void factor_launches(ddps_handle* h, cudaStream_t s) {
   launch_gather_rt_values(h->vals, h->rt_src, h->nrt, h->rt_val, s);
   h->launches++;
   const int64_t m = (int64_t)A.c.size();
-  if constexpr (std::is_same<T, double>::value) {
-    if (h->oz && m > 0) {  // cut the A operands of the tile ops into digits
-      Prof pr(h, DDPS_PROF_SPIKE_FWD, s);
-      launch_oz_units(h->rowptr, h->colind, h->vals, h->iperm, A.n, h->oz_work, h->oz_u, s);
-      h->launches += oz_units_launches();
-      for (int op = 0; op < 4; ++op) {
-        const int32_t* tf = op == OP_FWD_L21 ? h->tr_front : op == OP_FWD_LINV ? h->fk_front : h->tk_front;
-        const int32_t* tm = op == OP_FWD_L21 ? h->tr_m0 : op == OP_FWD_LINV ? h->fk_m0 : h->tk_m0;
-        const int32_t nt = op == OP_FWD_L21 ? h->tr_ptr.back() : op == OP_FWD_LINV ? h->fk_ptr.back() : h->tk_ptr.back();
-        if (nt > 0) {
-          launch_oz_pack(op, h->F, h->oz_u, tf, tm, h->tc_aoff[op], nt, std::max(h->tc_max_kt[op], 1), arena, h->atc, s);
-          h->launches += 2;
-        }
-      }
-    }
-  }
   if constexpr (std::is_same<T, float>::value) {
     if (h->tc_passes && m > 0) {  // pack the A operands of the tile ops and W of the fused fronts
       Prof pr(h, DDPS_PROF_SPIKE_FWD, s);
@@ -1813,8 +1787,7 @@ void build_sparse_forward(ddps_handle* h, const std::vector<int32_t>& kf,
   h->fz_ptr.assign(1, 0);
   h->zr_ptr.assign(1, 0);
   std::vector<int32_t> fz, zr;
-  const bool tc = !tc_off.empty();   // tiles with packed A operands
-  const bool fusing = h->tc_passes > 0;  // fused front products (tensor-core spikes)
+  const bool tc = !tc_off.empty();
   for (int64_t c = 0; c < nchunks; ++c) {
     uint8_t* act = active.data() + c * nf;
     for (int32_t b = 0; b < A.p; ++b) {
@@ -1824,12 +1797,12 @@ void build_sparse_forward(ddps_handle* h, const std::vector<int32_t>& kf,
           for (int32_t a = f; a >= 0 && !act[a]; a = A.f_parent[a]) act[a] = 1;
     }
     uint8_t* pl = pleaf.data() + c * nf;
-    if (fusing) {
+    if (tc) {
       for (int64_t f = 0; f < nf; ++f)
         if (act[f] || !fusedb[f]) zr.push_back((int32_t)f);
       h->zr_ptr.push_back((int64_t)zr.size());
     }
-    if (fusing)
+    if (tc)
       for (int64_t f = 0; f < nf; ++f) {
         if (!act[f] || !fused[f]) continue;
         bool child = false;
@@ -1864,7 +1837,7 @@ void build_sparse_forward(ddps_handle* h, const std::vector<int32_t>& kf,
     }
   }
   h->fw_active = dupload(h, active);
-  if (fusing) {
+  if (tc) {
     h->fw_pleaf = dupload(h, pleaf);
     h->zr_front = dupload(h, zr);
   }
@@ -1951,21 +1924,6 @@ void pack_ilu(ddps_handle* h, int64_t fs) {
   h->il_uval = dalloc_bytes(h, n * 4 * gu * fs);
   h->block_ptr = dupload(h, A.block_ptr);
   h->il_packed = true;
-}
-
-// Whether the FP64 spike products run in fixed point on the tensor cores: always the faster
-// (24^2, three blocks: 0.49 -> 0.45 ms a factorisation; 48^3, eight slabs: 278 -> 62), but the
-// digits take 14 bytes per entry of the factors: not past 24 GB, nor where what is left of the
-// device's memory (factors, G^ and panels are allocated) would not hold them and the vectors.
-bool oz_wins(const Analysis& A) {
-  int64_t bytes = 0;
-  for (size_t f = 0; f < A.f_k.size(); ++f) {
-    const int32_t k = A.f_k[f], r = A.f_m[f] - k, tk = (k + oz_tile_m() - 1) / oz_tile_m(), tr = (r + oz_tile_m() - 1) / oz_tile_m();
-    bytes += tk * (2 * oz_tile_bytes(k) + oz_tile_bytes(r)) + tr * oz_tile_bytes(k);
-  }
-  size_t left = 0, total = 0;
-  CK(cudaMemGetInfo(&left, &total));
-  return bytes <= (int64_t)24 << 30 && bytes + 40 * 8 * A.n + ((int64_t)1 << 30) <= (int64_t)left;
 }
 
 // Triangular inverses of the wide FP32 fronts from those of their diagonal blocks, two
@@ -2276,12 +2234,9 @@ void build_device(ddps_handle* h, const int32_t* rowptr, const int32_t* colind) 
                                      (int64_t)prec_size(h->opt.factor_prec));
   }
   {
+    const int BM = h->opt.factor_prec == DDPS_FP64 ? spike_tile_m<double>() : spike_tile_m<float>();
     const int sp = h->opt.spike_prec;
     const bool tcp = (sp == DDPS_BF16 || sp == DDPS_BF16X3) && m > 0 && !implicit;
-    h->oz = h->opt.factor_prec == DDPS_FP64 && m > 0 && !implicit && !A.ilu && oz_wins(A);
-    const int BM = h->oz                             ? oz_tile_m()
-                   : h->opt.factor_prec == DDPS_FP64 ? spike_tile_m<double>()
-                                                     : spike_tile_m<float>();
     const int passes = sp == DDPS_BF16X3 ? 3 : 1;
     const int64_t nfr = (int64_t)A.f_k.size();
     // fronts whose output rows fit one CTA take the fused products
@@ -2337,11 +2292,11 @@ void build_device(ddps_handle* h, const int32_t* rowptr, const int32_t* colind) 
     h->tr_front = dupload(h, rf);
     h->tr_m0 = dupload(h, rm);
     h->bz = dupload(h, bz);
-    std::vector<std::vector<int64_t>> tc_off_host(tcp || h->oz ? 4 : 0);
-    const int BK = tc_tile_bk();
-    if (tcp || h->oz) {
-      h->tc_passes = tcp ? passes : 0;
-      const int64_t bb = tc_a_block_bytes(passes);
+    std::vector<std::vector<int64_t>> tc_off_host(tcp ? 4 : 0);
+    if (tcp) {
+      h->tc_passes = passes;
+      const int BK = tc_tile_bk();
+      const int64_t bb = tc_a_block_bytes(h->tc_passes);
       int64_t run = 0;
       for (int op = 0; op < 4; ++op) {
         const std::vector<int32_t>& tf = op == OP_FWD_L21 ? rf : op == OP_FWD_LINV ? fkf : bkf;
@@ -2351,20 +2306,13 @@ void build_device(ddps_handle* h, const int32_t* rowptr, const int32_t* colind) 
           const int32_t K = op == OP_BWD_U12 ? rr : kk;
           const int32_t nk = (K + BK - 1) / BK;
           off[t] = run;
-          run += h->oz ? oz_tile_bytes(K) : nk * bb;
+          run += nk * bb;
           h->tc_max_kt[op] = std::max(h->tc_max_kt[op], nk);
         }
         h->tc_aoff[op] = dupload(h, off);
         tc_off_host[op] = off;
       }
       h->atc = (unsigned char*)dalloc_bytes(h, std::max<int64_t>(run, 16));
-      if (h->oz) {
-        h->oz_work = (int32_t*)dalloc_bytes(h, 4 * n * sizeof(int32_t));
-        h->oz_u.r = (int32_t*)dalloc_bytes(h, n * sizeof(int32_t));
-        h->oz_u.c = (int32_t*)dalloc_bytes(h, n * sizeof(int32_t));
-      }
-    }
-    if (tcp) {
       // packed W of the fused fronts
       std::vector<int64_t> wob(nfr, -1), wof(nfr, -1);
       std::vector<int32_t> pf;  // fused forward fronts

@@ -240,25 +240,6 @@ void launch_spike_gemm_tc(int op, int passes, DevFronts F, const int32_t* tile_f
                           const unsigned char* atc, int32_t ntiles, const int64_t* block_ncols,
                           int64_t j0, int32_t NR, float* X, float* Tb, long long* err,
                           int inject_wait, cudaStream_t s);
-// spike_oz.cu: the same ops for FP64 factors on the tensor cores, in fixed point (tiles of
-// oz_tile_m() rows; A packed once per factorisation, oz_tile_bytes(K) bytes per tile at
-// tile_aoff, 16-byte aligned).  A wait that runs out writes 2 into err[0].
-struct OzUnits {
-  int32_t *r, *c;  // exponents of the equations' and the unknowns' units (new indices)
-};
-// work: 4 n integers, 8-byte aligned.
-void launch_oz_units(const int32_t* rowptr, const int32_t* colind, const double* vals,
-                     const int32_t* iperm, int64_t n, int32_t* work, OzUnits U, cudaStream_t s);
-constexpr int oz_units_launches() { return 6; }
-constexpr int oz_tile_m() { return 32; }
-int64_t oz_tile_bytes(int K);
-void launch_oz_pack(int op, DevFronts F, OzUnits U, const int32_t* tile_front, const int32_t* tile_m0,
-                    const int64_t* tile_aoff, int32_t ntiles, int32_t max_kt, const double* arena,
-                    unsigned char* packed, cudaStream_t s);
-void launch_spike_gemm_oz(int op, DevFronts F, OzUnits U, const int32_t* tile_front, const int32_t* tile_m0,
-                          const int64_t* tile_aoff, const unsigned char* packed, int32_t ntiles,
-                          const int64_t* block_ncols, int64_t j0, int32_t NR, double* X, double* Tb,
-                          long long* err, cudaStream_t s);
 template <typename T>
 void launch_spike_gemm(int op, DevFronts F, const int32_t* tile_front, const int32_t* tile_m0,
                        int32_t ntiles, const T* arena, const int64_t* block_ncols, int64_t j0,

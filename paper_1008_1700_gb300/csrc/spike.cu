@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "launch.h"
 
@@ -28,8 +29,8 @@ struct Cfg<float> {
   static constexpr int BM = 128, BN = 128, BK = 8, TM = 8, TN = 8;
 };
 template <>
-struct Cfg<double> {
-  static constexpr int BM = 64, BN = 64, BK = 8, TM = 4, TN = 4;
+struct Cfg<double> {  // k_spike_gemm_fp64
+  static constexpr int BM = 32, BN = 128;
 };
 
 // T_f = [X rows of the pivots; 0] + sum over children of their update rows.
@@ -153,12 +154,13 @@ __global__ void __launch_bounds__(kThreads)
 // columns; A is a block of the front (column-major, leading dimension m,
 // triangular for the two inverse ops), B rows come from the panel or from the
 // front's working rows (gathered through the front's row list for OP_BWD_U12).
-template <typename T, int OP>
+template <int OP>
 __global__ void __launch_bounds__(kThreads)
     k_spike_gemm(DevFronts F, const int32_t* __restrict__ tile_front,
-                 const int32_t* __restrict__ tile_m0, const T* __restrict__ arena,
+                 const int32_t* __restrict__ tile_m0, const float* __restrict__ arena,
                  const int64_t* __restrict__ block_ncols, int64_t j0, int32_t NR,
-                 T* __restrict__ X, T* __restrict__ Tb) {
+                 float* __restrict__ X, float* __restrict__ Tb) {
+  using T = float;
   constexpr int BM = Cfg<T>::BM, BN = Cfg<T>::BN, BK = Cfg<T>::BK, TM = Cfg<T>::TM, TN = Cfg<T>::TN;
   __shared__ T As[BK][BM + 4];
   __shared__ T Bs[BK][BN + 4];
@@ -259,6 +261,103 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
+// The same products for FP64 factors, by FP64 FMAs, which run at 1/64 of the FP32 rate here:
+// bound by them, so the kernel spends no FMA on a zero.  A CTA takes 32 front rows times 128
+// panel columns, a warp 8 rows times 32 columns (a lane per column; A's entries are the same
+// for the whole warp).  A first pass over B finds each column's first and last entry that is
+// not zero: right-hand sides reach few of a front's rows, and a column begins where the
+// elimination met its first one.  A warp runs over the values of K between the first and the
+// last of its columns, and within its rows' part of a triangle.  The terms left out have an
+// exact zero of B or of the triangle as a factor, and the order of the others is that of a
+// sum over all of K.  48^3, eight slabs, FP64: forward and backward products 22.1 + 109 ms; over
+// all of K, in 64 x 64 tiles through shared memory, 54.7 + 207.
+template <int OP>
+__global__ void __launch_bounds__(512, 2)
+    k_spike_gemm_fp64(DevFronts F, const int32_t* __restrict__ tile_front,
+                      const int32_t* __restrict__ tile_m0, const double* __restrict__ arena,
+                      const int64_t* __restrict__ block_ncols, int64_t j0, int32_t NR,
+                      double* __restrict__ X, double* __restrict__ Tb) {
+  constexpr int BM = Cfg<double>::BM, BN = Cfg<double>::BN, R = 8;  // rows of a warp
+  __shared__ int first[BN], last[BN];
+  const int32_t f = tile_front[blockIdx.x];
+  const int32_t m0 = tile_m0[blockIdx.x];
+  const int n0 = blockIdx.y * BN;
+  const int64_t ncols = min((int64_t)NR, block_ncols[F.block[f]] - j0);
+  if (n0 >= ncols) return;
+  const int32_t k = F.k[f], m = F.m[f];
+  const int M = OP == OP_FWD_L21 ? m - k : k, K = OP == OP_BWD_U12 ? m - k : k;
+  const double* __restrict__ A =
+      arena + F.arena[f] + (OP == OP_FWD_L21 ? k : 0) + (OP == OP_BWD_U12 ? (int64_t)k * m : 0);
+  const int64_t row0 = F.row0[f], tb0 = F.idx_off[f];
+  const int32_t* __restrict__ idx = F.idx + tb0;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int c = (warp % (BN / 32)) * 32 + lane, part = warp / (BN / 32);
+  const bool live = n0 + c < ncols;
+  const double* Bp = ((OP == OP_FWD_L21 || OP == OP_BWD_U12) ? X : Tb) + n0 + c;
+  auto b_at = [&](int gk) -> double {
+    const int64_t row = OP == OP_FWD_L21 ? row0 + gk : OP == OP_BWD_U12 ? (int64_t)idx[k + gk] : tb0 + gk;
+    return live ? Bp[row * NR] : 0.0;
+  };
+  // the tile's part of a triangle
+  const int k0 = OP == OP_BWD_UINV ? m0 : 0, k1 = OP == OP_FWD_LINV ? min(K, m0 + BM) : K;
+  if (tid < BN) {
+    first[tid] = K;
+    last[tid] = -1;
+  }
+  __syncthreads();
+  int lo = K, hi = -1;
+#pragma unroll 8
+  for (int gk = k0 + part; gk < k1; gk += BM / R)
+    if (b_at(gk) != 0.0) {
+      lo = min(lo, gk);
+      hi = gk;
+    }
+  if (hi >= 0) {
+    atomicMin(&first[c], lo);
+    atomicMax(&last[c], hi);
+  }
+  __syncthreads();
+  lo = __reduce_min_sync(0xffffffffu, first[c]);
+  hi = __reduce_max_sync(0xffffffffu, last[c]) + 1;
+  const int i0 = m0 + part * R;
+  if (i0 >= M) return;
+  if (OP == OP_FWD_LINV) hi = min(hi, i0 + R);
+  if (OP == OP_BWD_UINV) lo = max(lo, i0);
+  double acc[R];
+#pragma unroll
+  for (int u = 0; u < R; ++u) acc[u] = 0.0;
+#pragma unroll 4
+  for (int gk = lo; gk < hi; ++gk) {
+    const double b = b_at(gk);
+#pragma unroll
+    for (int u = 0; u < R; ++u) {
+      const int i = i0 + u;
+      double a = A[min(i, M - 1) + (int64_t)gk * m];
+      if (OP == OP_FWD_LINV) a = i > gk ? a : i == gk ? 1.0 : 0.0;
+      if (OP == OP_BWD_UINV) a = i <= gk ? a : 0.0;
+      acc[u] = fma(a, b, acc[u]);
+    }
+  }
+  if (!live) return;
+  const double* cin = nullptr;
+  double* out;
+  if (OP == OP_FWD_LINV || OP == OP_BWD_UINV) {
+    out = X + (row0 + i0) * NR;
+  } else if (OP == OP_FWD_L21) {
+    out = Tb + (tb0 + k + i0) * NR;
+    cin = out;
+  } else {
+    out = Tb + (tb0 + i0) * NR;
+    cin = X + (row0 + i0) * NR;
+  }
+#pragma unroll
+  for (int u = 0; u < R; ++u) {
+    if (i0 + u >= M) break;
+    const int64_t o = (int64_t)u * NR + n0 + c;
+    out[o] = cin ? cin[o] - acc[u] : acc[u];
+  }
+}
+
 }  // namespace
 
 template <typename T>
@@ -290,23 +389,19 @@ void launch_spike_gemm(int op, DevFronts F, const int32_t* tile_front, const int
                        int32_t NR, T* X, T* Tb, cudaStream_t s) {
   if (ntiles <= 0) return;
   dim3 grid(ntiles, (NR + Cfg<T>::BN - 1) / Cfg<T>::BN);
-  switch (op) {
-    case OP_FWD_LINV:
-      k_spike_gemm<T, OP_FWD_LINV><<<grid, kThreads, 0, s>>>(F, tile_front, tile_m0, arena,
-                                                              block_ncols, j0, NR, X, Tb);
-      break;
-    case OP_FWD_L21:
-      k_spike_gemm<T, OP_FWD_L21><<<grid, kThreads, 0, s>>>(F, tile_front, tile_m0, arena,
-                                                             block_ncols, j0, NR, X, Tb);
-      break;
-    case OP_BWD_U12:
-      k_spike_gemm<T, OP_BWD_U12><<<grid, kThreads, 0, s>>>(F, tile_front, tile_m0, arena,
-                                                             block_ncols, j0, NR, X, Tb);
-      break;
-    default:
-      k_spike_gemm<T, OP_BWD_UINV><<<grid, kThreads, 0, s>>>(F, tile_front, tile_m0, arena,
-                                                              block_ncols, j0, NR, X, Tb);
-  }
+  auto run = [&](auto kern, int threads) {
+    kern<<<grid, threads, 0, s>>>(F, tile_front, tile_m0, arena, block_ncols, j0, NR, X, Tb);
+  };
+  if constexpr (std::is_same<T, double>::value)
+    run(op == OP_FWD_LINV  ? k_spike_gemm_fp64<OP_FWD_LINV>
+        : op == OP_FWD_L21 ? k_spike_gemm_fp64<OP_FWD_L21>
+        : op == OP_BWD_U12 ? k_spike_gemm_fp64<OP_BWD_U12>
+                           : k_spike_gemm_fp64<OP_BWD_UINV>, 512);
+  else
+    run(op == OP_FWD_LINV  ? k_spike_gemm<OP_FWD_LINV>
+        : op == OP_FWD_L21 ? k_spike_gemm<OP_FWD_L21>
+        : op == OP_BWD_U12 ? k_spike_gemm<OP_BWD_U12>
+                           : k_spike_gemm<OP_BWD_UINV>, kThreads);
 }
 
 #define DDPS_INST_SP(T)                                                                         \

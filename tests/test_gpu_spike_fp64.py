@@ -61,3 +61,91 @@ def test_ghat_residual(kind, size, q, units):
     bound = 3 * 3 * nb * 2.0 ** -53 * np.linalg.norm(np.abs(M) @ np.abs(X), axis=0)
     assert np.all(np.linalg.norm(res.astype(float), axis=0) <= bound)
     S.close()
+
+
+def _ghat(M, R):
+    """G^ = M^-1 R of a block whose rows are all interface rows; R: one column per coupling
+    unknown, with an entry in every column."""
+    nb, q = R.shape
+    C = np.zeros((q, nb))
+    C[np.arange(nb) % q, np.arange(nb)] = 0.01
+    A = sp.csr_matrix(np.block([[M, R], [C, np.eye(q) * 10.0]]))
+    A.sort_indices()
+    S = Solver(A.indptr, A.indices, np.array([0, nb, nb + q]), **FP64)
+    S.factor(dev(A.data))
+    q0, q1, cols = S.ghat_layout(0)
+    c = S.interface()
+    assert (q0, q1) == (0, nb) and np.array_equal(c[q0:q1], np.arange(nb))
+    X = np.zeros((nb, q))
+    X[:, c[cols] - nb] = S.ghat_block(0)
+    S.close()
+    return X
+
+
+@pytest.mark.parametrize("weak", [1e-12, 1e-17, 1e-40, 1e-300])
+@pytest.mark.parametrize("kind", ["half", "band"])
+def test_weak_couplings_in_part_of_a_block(kind, weak):
+    """Couplings that are numerically nothing, in half of the rows or far from the diagonal,
+    cost the other rows no digits."""
+    rng = np.random.default_rng(7)
+    nb, q = 130, 140
+    M = rng.uniform(-1.0, 1.0, (nb, nb))
+    if kind == "half":
+        M[nb // 2:] *= weak
+    else:
+        far = np.abs(np.subtract.outer(np.arange(nb), np.arange(nb)))
+        M[far > 3] *= weak
+    np.fill_diagonal(M, 0.0)
+    np.fill_diagonal(M, 1.5 * np.abs(M).sum(axis=1) + 1.0)
+    R = rng.uniform(-1.0, 1.0, (nb, q))
+    X = _ghat(M, R)
+    res = np.longdouble(M) @ X - R
+    # as in test_ghat_residual
+    bound = 3 * 3 * nb * 2.0 ** -53 * np.linalg.norm(np.abs(M) @ np.abs(X), axis=0)
+    assert np.all(np.linalg.norm(res.astype(float), axis=0) <= bound)
+
+
+def test_small_entries_keep_their_digits():
+    """A strongly dominant M-matrix on a 7-point grid: every sum of the factorisation and of
+    the sweeps has terms of one sign but for the pivots, which lose a few percent, so each
+    entry of G^ carries a relative error of the roundings it passed through, at most nb in
+    each of the LU, the inverses and the two sweeps -- also where it is 2^-140 of the
+    column's largest."""
+    n1 = 7
+    line = sp.diags([1.0] * 2, [-1, 1], shape=(n1, n1))
+    e = sp.identity(n1)
+    P = (sp.kron(sp.kron(line, e), e) + sp.kron(sp.kron(e, line), e) + sp.kron(sp.kron(e, e), line))
+    rng = np.random.default_rng(3)
+    M = -P.toarray() * rng.uniform(0.5, 1.0, P.shape) * 2.0 ** -7 + np.eye(n1 ** 3)
+    nb, q = len(M), 40
+    R = np.zeros((nb, q))
+    R[rng.choice(nb, q, replace=False), np.arange(q)] = 1.0
+    X = _ghat(M, R)
+    W = np.concatenate([M, R], axis=1).astype(np.longdouble)
+    for j in range(nb):  # Gauss-Jordan without exchanges: entries of one sign here too
+        W[j] /= W[j, j]
+        col = W[:, j].copy()
+        col[j] = 0
+        W -= np.outer(col, W[j])
+    ref = W[:, nb:]
+    assert ref.min() > 0 and float(ref.min()) < 2.0 ** -100
+    assert np.max(np.abs(X - ref) / ref) <= 1.2 * 4 * (nb + 1) * 2.0 ** -53
+
+
+def test_overflowed_inverse_is_not_a_number():
+    """An equation in units of 1e-310, eliminated last: its pivot passes the test against the
+    row's norm, but the pivot's reciprocal overflows.  G^ is not finite there."""
+    rng = np.random.default_rng(5)
+    nb, q = 8, 3
+    M = rng.uniform(-1.0, 1.0, (nb, nb))
+    np.fill_diagonal(M, 10.0)
+    R = rng.uniform(0.5, 1.0, (nb, q))
+    C = np.full((q, nb), 0.01)
+    rows = sp.csr_matrix(np.block([[M, R], [C, np.eye(q) * 10.0]]))
+    _, perm, _ = N.ddps_symbolic(rows.indptr, rows.indices, np.array([0, nb, nb + q]),
+                                 values=rows.data, options=N.default_options(**FP64))
+    last = int(perm[nb - 1])
+    M[last] *= 1e-310
+    R[last] *= 1e-310
+    X = _ghat(M, R)
+    assert not np.isfinite(X[last]).any()
