@@ -2392,6 +2392,9 @@ void build_device(ddps_handle* h, const int32_t* rowptr, const int32_t* colind) 
   for (void** pp : inner) *pp = dalloc_bytes(h, std::max<int64_t>(m, 1) * (int64_t)is);
   h->sc_out = dalloc<KScal>(h, h->nseg);
   h->sc_in = dalloc<KScal>(h, h->nseg);
+  // a system without reduced rows has no part in the inner iteration in one launch
+  // (launch_inner_cluster): its scalars stay zero
+  CK(cudaMemset(h->sc_in, 0, sizeof(KScal) * h->nseg));
   CK(cudaMallocHost((void**)&h->hsc_out, sizeof(KScal) * h->nseg));
   CK(cudaMallocHost((void**)&h->hsc_in, sizeof(KScal) * h->nseg));
   CK(cudaMallocHost((void**)&h->hstage, sizeof(KScal) * h->nseg * kStageSlots));

@@ -3,6 +3,8 @@ one block (c is empty and Fig. 3 is one LU solve), everything dropped (c is
 empty, DDPS is block Jacobi inside the Krylov loop), ragged partitions with
 one-row blocks, a tiny system, the identity, and batches that mix these."""
 
+import ctypes
+
 import numpy as np
 import pytest
 import scipy.sparse as sp
@@ -233,3 +235,38 @@ def test_dense_front_edges(rows, prec):
     # the inverses and the two triangular products
     assert np.linalg.norm(D @ x - y[:rows]) <= 3 * 4 * (rows + 1) * u * np.linalg.norm(np.abs(D) @ np.abs(x))
     S.close()
+
+
+@pytest.mark.parametrize("form", ["fp64", "mixed"])
+def test_statistics_of_a_batch_with_an_uncoupled_system(form):
+    """A system without coupling columns takes no part in the reduced solve: the counts
+    returned are those of the coupled one alone, whatever the device memory held before."""
+    opts = dict(FP64 if form == "fp64" else MIXED_TC, tol_out=1e-10, tol_in=1e-6)
+    a, b = W.small_random_band(300, 1, 30, seed=8), W.small_convdiff_2d(10, 10)
+
+    def run(probs):
+        S = Solver.from_systems([(p.rowptr, p.colind, p.values, p.block_ptr) for p in probs], **opts)
+        S.factor(dev(S.values_host))
+        g = dev(np.linspace(1.0, 2.0, S.m))
+        z = host(S.reduced_solve(g))
+        info = S.solve(dev(np.concatenate([p.f for p in probs])))[1]
+        S.close()
+        return z, info
+    z1, alone = run([b])
+    # every other one of many small blocks full of bytes 0x41 is given back: the next handle's
+    # small allocations come from these (memory of a wholly free region is cleared)
+    rt = ctypes.CDLL("libcudart.so")
+    junk = [ctypes.c_void_p() for _ in range(20000)]
+    for q in junk:
+        assert rt.cudaMalloc(ctypes.byref(q), ctypes.c_size_t(512)) == 0
+        assert rt.cudaMemset(q, 0x41, ctypes.c_size_t(512)) == 0
+    for q in junk[::2]:
+        assert rt.cudaFree(q) == 0
+    z2, both = run([a, b])
+    for q in junk[1::2]:
+        assert rt.cudaFree(q) == 0
+    assert alone["guess_used"] == both["guess_used"] == 0
+    assert both["first_inner_iters"] == alone["first_inner_iters"]
+    # the uncoupled system may add outer iterations, in which the coupled one takes none
+    assert both["inner_iterations"] == alone["inner_iterations"]
+    assert np.array_equal(z1, z2)
