@@ -226,8 +226,9 @@ ddps_status ddps_factor_host(ddps_handle* h, const double* values_host, void* st
  *   nrhs  number of right-hand sides (>= 1), solved with the same factors (the
  *         factor phase needs no right-hand side, Sec. 3): one after the other,
  *         or up to four together (stored G^ of at most 32 bits, iterative reduced
- *         solve of a system too large for one cluster, no reduced guess set; the
- *         first such solve allocates their vectors, 4 GB at most)
+ *         solve of a system too large for one cluster, no reduced guess set; a
+ *         solve of more of them than any before allocates their vectors, 4 GB at
+ *         most, which the handle keeps; where they don't fit, one after the other)
  *   x0    device float64[n * nrhs] initial guesses, or NULL for x0 = 0; a
  *         guess that already meets tol_out is returned after no iteration
  *   info  host, may be NULL: iterations are the largest over the right-hand

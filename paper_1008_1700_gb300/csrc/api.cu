@@ -237,9 +237,13 @@ struct ddps_handle : SolveWork {
   double *im_q = nullptr, *im_g = nullptr;  // implicit G^: R~ v and D~^-1 R~ v
   // host-buffer entry points stage f and x here
   double *io_f = nullptr, *io_x = nullptr;
-  // several right-hand sides together (kMaxWide at most; allocated by the first such solve)
+  // several right-hand sides together (wide_cap of them, kMaxWide at most; allocated by the first
+  // solve of so many)
   SolveWork wide;
-  bool wide_ok = false, wide_failed = false;
+  int wide_cap = 0;
+  bool wide_failed = false;
+  std::vector<void*> wide_allocs;
+  int64_t wide_bytes = 0;
   cudaGraphExec_t wide_inner[kMaxWide + 1] = {}, wide_sweeps[kMaxWide + 1] = {};
   int64_t wide_inner_launches[kMaxWide + 1] = {}, wide_sweeps_launches[kMaxWide + 1] = {};
   std::vector<double> rhs_iters;  // inner iterations of the last reduced solves, per right-hand side
@@ -1627,11 +1631,31 @@ int wide_width(ddps_handle* h, int32_t nrhs) {
 
 constexpr int64_t kWideBytes = (int64_t)4 << 30;  // most memory taken for the wide vectors
 
-// The wide workspace, in one allocation; false if it is too large or there is no room.
-bool ensure_wide(ddps_handle* h) {
-  if (h->wide_ok) return true;
+// Gives the wide workspace and its graphs back (no solve is in flight: solves end synchronised).
+void release_wide(ddps_handle* h) {
+  for (int W = 2; W <= kMaxWide; ++W) {
+    if (h->wide_inner[W]) cudaGraphExecDestroy(h->wide_inner[W]);
+    if (h->wide_sweeps[W]) cudaGraphExecDestroy(h->wide_sweeps[W]);
+    h->wide_inner[W] = h->wide_sweeps[W] = nullptr;
+  }
+  for (void* p : h->wide_allocs) cudaFree(p);
+  if (h->wide.hsc_out) cudaFreeHost(h->wide.hsc_out);
+  if (h->wide.hsc_in) cudaFreeHost(h->wide.hsc_in);
+  if (h->wide.hstage) cudaFreeHost(h->wide.hstage);
+  h->wide_allocs.clear();
+  h->bytes -= h->wide_bytes;
+  h->wide_bytes = 0;
+  h->wide = SolveWork{};
+  h->wide_cap = 0;
+}
+
+// The wide workspace for W right-hand sides, its vectors in one allocation; false, and nothing
+// held, if it is too large or there is no room.
+bool ensure_wide(ddps_handle* h, int W) {
+  if (h->wide_cap >= W) return true;
+  release_wide(h);
   const Analysis& A = h->A;
-  const int64_t W = kMaxWide, n = A.n, m = (int64_t)A.c.size(), ns = A.nsys * W;
+  const int64_t n = A.n, m = (int64_t)A.c.size(), ns = A.nsys * W;
   const int64_t fs = (int64_t)prec_size(h->opt.factor_prec), is = (int64_t)prec_size(h->opt.inner_prec);
   auto up = [](int64_t b) { return (b + 255) / 256 * 256; };
   const int64_t bn = up(W * n * 8), bm = up(W * m * 8), bi = up(W * m * is), bw = up(W * n * fs),
@@ -1642,6 +1666,13 @@ bool ensure_wide(ddps_handle* h) {
     h->wide_failed = true;
     return false;
   }
+  const size_t before = h->allocs.size();
+  const int64_t bytes0 = h->bytes;
+  auto own = [&]() {  // the allocations made here
+    h->wide_allocs.assign(h->allocs.begin() + before, h->allocs.end());
+    h->allocs.resize(before);
+    h->wide_bytes = h->bytes - bytes0;
+  };
   try {
     char* p = (char*)dalloc_bytes(h, total);
     auto take = [&](int64_t b) {
@@ -1677,10 +1708,13 @@ bool ensure_wide(ddps_handle* h) {
     k.hsc = k.hsc_out;
   } catch (const Fail&) {  // one after the other then
     cudaGetLastError();
+    own();
+    release_wide(h);
     h->wide_failed = true;
     return false;
   }
-  h->wide_ok = true;
+  own();
+  h->wide_cap = W;
   return true;
 }
 
@@ -1694,8 +1728,8 @@ struct WideScope {
     k.width = W;
     k.nseg = W * h->A.nsys;
     k.Sn.nseg = k.Sm.nseg = k.nseg;
-    k.Sn.nchunks = k.Sn.nchunks / kMaxWide * W;
-    k.Sm.nchunks = k.Sm.nchunks / kMaxWide * W;
+    k.Sn.nchunks = k.Sn.nchunks / h->wide_cap * W;
+    k.Sm.nchunks = k.Sm.nchunks / h->wide_cap * W;
     k.g_inner = h->wide_inner[W];
     k.g_inner_launches = h->wide_inner_launches[W];
     k.g_sweeps = h->wide_sweeps[W];
@@ -2698,7 +2732,7 @@ ddps_status ddps_solve(ddps_handle* h, const double* f, double* x, int32_t nrhs,
     ddps_solve_info acc{}, one{};
     for (int32_t j = 0, W = 1; j < nrhs; j += W) {
       W = wide_width(h, nrhs - j);
-      if (W > 1 && !ensure_wide(h)) W = 1;
+      if (W > 1 && !ensure_wide(h, W)) W = 1;
       ddps_status st;
       if (W > 1) {
         WideScope scope(h, W);
@@ -3013,18 +3047,12 @@ ddps_status ddps_destroy(ddps_handle* h) {
     cudaStreamDestroy(h->gstream);
   }
   for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
+  release_wide(h);
   for (void* p : h->allocs) cudaFree(p);
   if (h->herr) cudaFreeHost(h->herr);
   if (h->hsc_out) cudaFreeHost(h->hsc_out);
   if (h->hsc_in) cudaFreeHost(h->hsc_in);
   if (h->hstage) cudaFreeHost(h->hstage);
-  if (h->wide.hsc_out) cudaFreeHost(h->wide.hsc_out);
-  if (h->wide.hsc_in) cudaFreeHost(h->wide.hsc_in);
-  if (h->wide.hstage) cudaFreeHost(h->wide.hstage);
-  for (int W = 2; W <= kMaxWide; ++W) {
-    if (h->wide_inner[W]) cudaGraphExecDestroy(h->wide_inner[W]);
-    if (h->wide_sweeps[W]) cudaGraphExecDestroy(h->wide_sweeps[W]);
-  }
   if (h->any_host) cudaFreeHost(h->any_host);
   delete h;
   return DDPS_OK;

@@ -51,3 +51,27 @@ def test_together_equals_one_at_a_time(form, nrhs, systems):
     y, again = S.solve(dev(f), x0=x)
     assert again["precond_applies"] == 0 and np.array_equal(host(y), host(x))
     S.close()
+
+
+def test_workspace_is_for_the_right_hand_sides_asked_for():
+    """Two right-hand sides take room for two; four, later, for four and no more; solutions
+    and counts after the workspace has grown are those of a new handle."""
+    P = W.small_convdiff_3d(27, [9, 8, 10])
+    f = np.random.default_rng(4).uniform(-1.0, 1.0, (4, P.n))
+    held = lambda S: N.ddps_get_sizes(S.h)["device_bytes"]
+    S = make_solver(P, **FORMS["fp16"])
+    b0 = held(S)
+    x2, _ = S.solve(dev(f[:2]))
+    b2 = held(S) - b0
+    x4, i4 = S.solve(dev(f))
+    b4 = held(S) - b0
+    assert 0 < b2 <= 0.55 * b4
+    again, _ = S.solve(dev(f[:2]))
+    assert held(S) - b0 == b4 and np.array_equal(host(again), host(x2))
+    T = make_solver(P, **FORMS["fp16"])
+    c0 = held(T)
+    y4, j4 = T.solve(dev(f))
+    assert held(T) - c0 == b4 and np.array_equal(host(y4), host(x4))
+    assert i4["inner_iterations"] == j4["inner_iterations"]
+    S.close()
+    T.close()
