@@ -1945,6 +1945,22 @@ void pack_ilu(ddps_handle* h, int64_t fs) {
     h->il_max_rows = std::max(h->il_max_rows, A.block_ptr[b + 1] - A.block_ptr[b]);
   }
   h->il_max_level = std::max(lo.max_level, up.max_level);
+  {
+    const int nt = ilu_threads(h->il_max_level);
+    std::vector<int32_t> steps(A.p, 0);
+    std::vector<int64_t> rounds(A.p, 0);
+    for (const Host* H : {&lo, &up})
+      for (int32_t b = 0; b < A.p; ++b)
+        for (int32_t l = H->off[b]; l + 1 < H->off[b + 1]; ++l) {
+          ++steps[b];
+          rounds[b] += (H->lev[l + 1] - H->lev[l] + nt - 1) / nt;
+        }
+    const int32_t launches = 2 + (int32_t)(A.il_lf_ptr.size() - 1 + A.il_lb_ptr.size() - 1);
+    auto one = fs == 8 ? ilu_one_launch<double> : ilu_one_launch<float>;
+    if (!one(A.p, h->il_max_rows, h->il_max_starts, std::max(gl, gu), nt, steps.data(), rounds.data(),
+             launches))
+      return;
+  }
   auto upload = [&](const Host& H, int32_t groups, IluSweep& S) {
     S.col = dupload(h, H.col);
     S.lev = dupload(h, H.lev);

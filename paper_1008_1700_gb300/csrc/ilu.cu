@@ -292,15 +292,17 @@ void launch_ilu_pack(const T* a, const int32_t* src, int64_t cnt, T* out, cudaSt
 }
 
 constexpr size_t kIluSmem = 220 * 1024;
+// level starts in shared memory; very many of them stay in global memory
+static size_t lev_bytes(int32_t max_starts) {
+  const size_t lev = ((size_t)max_starts * 4 + 15) / 16 * 16;
+  return lev > kIluSmem / 8 ? 0 : lev;
+}
 
 template <typename T, int Q, int NT>
 static void launch_solve(int32_t nblocks, int64_t max_rows, int32_t max_starts, const IluSweep& L,
                          const IluSweep& U, const T* lval, const T* uval, int64_t n,
                          const int64_t* block_ptr, const double* y, T* w, double* g, cudaStream_t s) {
-  // level starts and vector in shared memory; very many levels stay in global memory
-  size_t lev = ((size_t)max_starts * 4 + 15) / 16 * 16;
-  if (lev > kIluSmem / 8) lev = 0;
-  const size_t ring = sizeof(IluRing<T, Q, NT>);
+  const size_t lev = lev_bytes(max_starts), ring = sizeof(IluRing<T, Q, NT>);
   const size_t sm = ring + lev + (size_t)max_rows * sizeof(T);
   if (sm <= kIluSmem) {
     record_launch_error(cudaFuncSetAttribute(k_ilu_solve<T, Q, NT, true>,
@@ -315,6 +317,31 @@ static void launch_solve(int32_t nblocks, int64_t max_rows, int32_t max_starts, 
   }
 }
 
+// A CTA walks its block alone: a step of at most as many rows as it has threads takes 0.4 us
+// (vector in shared memory) or 1.5 (in global memory), every further round of a wider level,
+// whose rows were not copied ahead, 1 or 2.6; FP64 half as much again.  A launch per level
+// takes 5.5 us, and its rows spread over all SMs.  Measured, one launch against a launch per
+// level in us, FP32: 64^3 in 16 slabs 88 / 1,434, in two 1,240 / 1,679; 96^3 in eight 1,346 /
+// 2,354, in two 4,579 / 2,709; 128^3 in two 10,956 / 4,037; a 1000 x 1000 grid in two 4,392 /
+// 16,255; eight levels of 62,500 rows 2,805 / 67, of 625 rows 21 / 46.
+template <typename T>
+bool ilu_one_launch(int32_t nblocks, int64_t max_rows, int32_t max_starts, int32_t groups,
+                    int threads, const int32_t* steps, const int64_t* rounds, int32_t launches) {
+  const size_t ring = groups <= 1 ? (threads == 256 ? sizeof(IluRing<T, 1, 256>) : sizeof(IluRing<T, 1, 512>))
+                                  : (threads == 256 ? sizeof(IluRing<T, 2, 256>) : sizeof(IluRing<T, 2, 512>));
+  size_t sm = ring + lev_bytes(max_starts) + (size_t)max_rows * sizeof(T);
+  const bool shared = sm <= kIluSmem;
+  if (!shared) sm = ring + lev_bytes(max_starts);
+  const double step = shared ? 0.4 : 1.5, more = shared ? 1.0 : 2.6;
+  double longest = 0.0;
+  for (int32_t b = 0; b < nblocks; ++b)
+    longest = std::max(longest, step * steps[b] + more * (double)(rounds[b] - steps[b]));
+  if (sizeof(T) == 8) longest *= 1.5;
+  const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(1024 / threads, 227 * 1024 / (sm + 1024)));
+  const int at_once = per_sm * device_sm_count();
+  return longest * ((nblocks + at_once - 1) / at_once) <= 5.5 * launches;
+}
+
 // max_level: rows of the widest level of a block.  256 threads while two rounds
 // cover it (a barrier of eight warps is cheaper), else 512; three entries a row in the
 // ring for the 5- and 7-point grids, else seven.
@@ -323,7 +350,7 @@ void launch_ilu_solve(int32_t nblocks, int64_t max_rows, int32_t max_level, int3
                       const IluSweep& L, const IluSweep& U, const T* lval, const T* uval, int64_t n,
                       const int64_t* block_ptr, const double* y, T* w, double* g, cudaStream_t s) {
   auto run = [&](auto fn) { fn(nblocks, max_rows, max_starts, L, U, lval, uval, n, block_ptr, y, w, g, s); };
-  const bool narrow = std::max(L.groups, U.groups) <= 1, small = max_level <= 512;
+  const bool narrow = std::max(L.groups, U.groups) <= 1, small = ilu_threads(max_level) == 256;
   if (narrow)
     run(small ? launch_solve<T, 1, 256> : launch_solve<T, 1, 512>);
   else
@@ -334,6 +361,8 @@ void launch_ilu_solve(int32_t nblocks, int64_t max_rows, int32_t max_level, int3
   template void launch_ilu0_level<T>(const int32_t*, int32_t, const IluDev&, T*, const double*, \
                                      double, long long*, cudaStream_t);                         \
   template void launch_ilu_pack<T>(const T*, const int32_t*, int64_t, T*, cudaStream_t);         \
+  template bool ilu_one_launch<T>(int32_t, int64_t, int32_t, int32_t, int, const int32_t*,       \
+                                  const int64_t*, int32_t);                                      \
   template void launch_ilu_solve<T>(int32_t, int64_t, int32_t, int32_t, const IluSweep&,         \
                                     const IluSweep&,                                             \
                                     const T*, const T*, int64_t, const int64_t*,                 \

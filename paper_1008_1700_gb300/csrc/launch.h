@@ -104,6 +104,14 @@ struct IluSweep {
 // out[i] = a[src[i]], 0 where src[i] < 0
 template <typename T>
 void launch_ilu_pack(const T* a, const int32_t* src, int64_t cnt, T* out, cudaStream_t s);
+// Threads of a CTA of launch_ilu_solve, by the rows of the widest level of a block.
+inline int ilu_threads(int32_t max_level) { return max_level <= 512 ? 256 : 512; }
+// Whether launch_ilu_solve takes less time than `launches` launches of launch_ilu_vec_level and
+// the permutations: steps, rounds: per block, its levels and the rounds of `threads` rows they
+// take; groups: packed groups of a row.
+template <typename T>
+bool ilu_one_launch(int32_t nblocks, int64_t max_rows, int32_t max_starts, int32_t groups,
+                    int threads, const int32_t* steps, const int64_t* rounds, int32_t launches);
 // g = (L~ U~)^-1 y, both sweeps of all blocks in one launch; w: n entries of work;
 // max_rows, max_level, max_starts: the largest block, level, and number of level
 // starts of a block's two sweeps

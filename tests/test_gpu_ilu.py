@@ -6,6 +6,7 @@ reaches the solution of A x = f."""
 
 import numpy as np
 import pytest
+import scipy.sparse as sp
 
 import workloads as W
 from gpu_helpers import dev, host, make_solver, relerr
@@ -107,3 +108,61 @@ def test_ilu_one_launch_solves(name, make):
     S = make_solver(P, **ILU64)
     assert relerr(host(S.block_solve(dev(y))), o.block_solve(y)) <= 1e-12
     S.close()
+
+
+def _launches(S, y):
+    n0 = S.launch_count()
+    g = host(S.block_solve(dev(y)))
+    return g, S.launch_count() - n0
+
+
+@pytest.mark.parametrize("prec,bound", [(N.DDPS_FP64, 1e-12), (N.DDPS_FP32, 2e-5)])
+@pytest.mark.parametrize("n,p,one", [(60000, 2, False), (60000, 100, True)])
+def test_ilu_block_solve_route_by_the_width_of_the_levels(n, p, one, prec, bound):
+    """Few levels of thousands of rows in two blocks take a launch per level, which spreads
+    their rows over the GPU; the same levels in many blocks take one launch.  The blocks are
+    lower triangular, so ILU(0) is exact."""
+    rng = np.random.default_rng(p)
+    bs, levels = n // p, 8
+    row = np.repeat(np.arange(n), 3)
+    level = row % bs * levels // bs
+    row, level = row[level > 0], level[level > 0]
+    col = row - row % bs + (level - 1) * bs // levels + rng.integers(0, bs // levels - 1, len(row))
+    A = sp.csr_matrix((rng.uniform(-0.3, 0.3, len(row)), (row, col)), shape=(n, n))
+    A = A + 2.0 * sp.identity(n)
+    A = A + sp.csr_matrix(([0.1], ([0], [n - 1])), shape=(n, n))  # blocks coupled by one entry
+    A = sp.csr_matrix(A)
+    A.sort_indices()
+    S = Solver(A.indptr, A.indices, np.arange(p + 1) * bs, **dict(ILU64 if prec == N.DDPS_FP64 else ILU32))
+    S.factor(dev(A.data))
+    y = rng.standard_normal(n)
+    g, launches = _launches(S, y)
+    D = sp.csr_matrix(sp.tril(A))
+    assert relerr(D @ g, y) <= bound
+    assert (launches == 1) == one, launches
+    S.close()
+
+
+def test_ilu_block_solve_of_an_arrow():
+    """A row and a column of full width in every block: rows are not padded to the widest, the
+    sweeps take a launch per level."""
+    n, p = 600, 2
+    rng = np.random.default_rng(2)
+    A = sp.lil_matrix(sp.diags([rng.uniform(-1, 1, n - 1), np.full(n, 500.0), rng.uniform(-1, 1, n - 1)],
+                               [-1, 0, 1]))
+    for b in range(p):
+        r0, r1 = b * n // p, (b + 1) * n // p
+        A[r1 - 1, r0:r1 - 1] = rng.uniform(-1, 1, r1 - r0 - 1)
+        A[r0:r1 - 1, r1 - 1] = rng.uniform(-1, 1, (r1 - r0 - 1, 1))
+    A = sp.csr_matrix(A)
+    A.sort_indices()
+    cuts = np.arange(p + 1, dtype=np.int64) * (n // p)
+    o = DDPSOracle(n, A.indptr.astype(np.int32), A.indices.astype(np.int32), A.data, cuts, factor="ilu0")
+    y = rng.standard_normal(n)
+    for opts, bound in ((ILU64, 1e-12), (ILU32, 2e-5)):
+        S = Solver(A.indptr, A.indices, cuts, **opts)
+        S.factor(dev(A.data))
+        g, launches = _launches(S, y)
+        assert relerr(g, o.block_solve(y)) <= bound
+        assert launches > 100
+        S.close()
