@@ -11,7 +11,7 @@
 // sums through distributed shared memory, one cluster barrier per reduction.  The
 // steps are those of the loop: products accumulate in FP32 (FP64 for FP64 storage),
 // vectors are rounded to the inner precision after each update, sums and scalars are
-// kept to about 48 bits or more (see Pair).  Sums are taken over threads, warps and
+// kept to FP64 or more (see Tri).  Sums are taken over threads, warps and
 // CTAs in a fixed order: two solves are bitwise equal.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -24,6 +24,7 @@
 
 #include "inner_cluster.h"
 #include "launch.h"
+#include "tri.h"
 
 namespace ddps {
 namespace cg = cooperative_groups;
@@ -89,75 +90,22 @@ struct Vec<__nv_bfloat16> {
   }
 };
 
-// Scalars and sums.  FP64 vectors take FP64.  For FP32 vectors they are unevaluated
-// pairs of floats (hi + lo, about 48 bits; products by fused multiply-add, sums by
-// Knuth's two-sum), because the FP64 pipe runs a warp instruction in 64 cycles here:
-// with FP64 sums, scalars and updates an iteration of a 384-row system took 18 us,
-// with pairs 12 (and 7.8 with fewer barriers, too).  Pairs have FP32's range, so the
-// system is scaled by the power of two that brings ||g|| to [1, 2).
-struct Pair {
-  float hi, lo;
-};
-__device__ __forceinline__ Pair two_sum(float a, float b) {
-  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
-  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+// Scalars and sums.  FP64 vectors take FP64.  For FP32 vectors they are unevaluated sums of
+// three floats (tri.h: about 70 bits, more than FP64 holds), because the FP64 pipe runs a warp
+// instruction in 64 cycles here: with FP64 sums, scalars and updates an iteration of a 384-row
+// system took 18 us at first, with pairs of floats (48 bits) 12, and 7.8 with fewer barriers,
+// too; the third float adds 1.1.  They have FP32's range, so the system is scaled by the power of
+// two that brings ||g|| to [2^20, 2^21): squares of vectors up to 10^13 ||g|| stay finite, and
+// those of 10^-17 ||g|| keep FP64's digits.
+__device__ __forceinline__ Tri shfl_xor(Tri x, int o) {
+  return {__shfl_xor_sync(0xffffffffu, x.h, o), __shfl_xor_sync(0xffffffffu, x.m, o),
+          __shfl_xor_sync(0xffffffffu, x.l, o)};
 }
-__device__ __forceinline__ Pair norm2(float hi, float lo) {
-  const float s = __fadd_rn(hi, lo);
-  return {s, __fsub_rn(lo, __fsub_rn(s, hi))};
-}
-__device__ __forceinline__ Pair add(Pair x, Pair y) {
-  const Pair s = two_sum(x.hi, y.hi);
-  return norm2(s.hi, __fadd_rn(s.lo, __fadd_rn(x.lo, y.lo)));
-}
-// running sums: the low part is not folded back (it stays below 2^-20 of hi's terms)
-__device__ __forceinline__ Pair sum(Pair x, Pair y) {
-  const Pair s = two_sum(x.hi, y.hi);
-  return {s.hi, __fadd_rn(s.lo, __fadd_rn(x.lo, y.lo))};
-}
-__device__ __forceinline__ Pair mul(float a, float b) {
-  const float p = __fmul_rn(a, b);
-  return {p, __fmaf_rn(a, b, -p)};
-}
-__device__ __forceinline__ Pair mul(Pair s, float b) {
-  const float p = __fmul_rn(s.hi, b);
-  return {p, __fmaf_rn(s.lo, b, __fmaf_rn(s.hi, b, -p))};
-}
-__device__ __forceinline__ Pair mul(Pair s, Pair b) {
-  const float p = __fmul_rn(s.hi, b.hi);
-  return norm2(p, __fmaf_rn(s.hi, b.lo, __fmaf_rn(s.lo, b.hi, __fmaf_rn(s.hi, b.hi, -p))));
-}
-__device__ __forceinline__ Pair neg(Pair x) { return {-x.hi, -x.lo}; }
-__device__ __forceinline__ Pair add(float a, Pair x) {
-  const Pair s = two_sum(a, x.hi);
-  return norm2(s.hi, __fadd_rn(s.lo, x.lo));
-}
-// quotient from two single-precision quotients: the second one of the remainder
-__device__ __forceinline__ Pair quot(Pair a, Pair b) {
-  const float q = a.hi / b.hi;
-  const Pair r = add(a, neg(mul(b, q)));
-  return norm2(q, r.hi / b.hi);
-}
-__device__ __forceinline__ float value(Pair x) { return x.hi; }
-__device__ __forceinline__ bool less(Pair a, Pair b) {
-  return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo);
-}
-__device__ __forceinline__ Pair shfl_xor(Pair x, int o) {
-  return {__shfl_xor_sync(0xffffffffu, x.hi, o), __shfl_xor_sync(0xffffffffu, x.lo, o)};
-}
-__device__ __forceinline__ Pair bcast(Pair x) {
-  return {__shfl_sync(0xffffffffu, x.hi, 0), __shfl_sync(0xffffffffu, x.lo, 0)};
+__device__ __forceinline__ Tri bcast(Tri x) {
+  return {__shfl_sync(0xffffffffu, x.h, 0), __shfl_sync(0xffffffffu, x.m, 0),
+          __shfl_sync(0xffffffffu, x.l, 0)};
 }
 __device__ __forceinline__ double bcast(double x) { return __shfl_sync(0xffffffffu, x, 0); }
-__device__ __forceinline__ Pair settle(Pair x) { return norm2(x.hi, x.lo); }
-__device__ __forceinline__ double add(double x, double y) { return x + y; }
-__device__ __forceinline__ double sum(double x, double y) { return x + y; }
-__device__ __forceinline__ double settle(double x) { return x; }
-__device__ __forceinline__ double mul(double a, double b) { return a * b; }
-__device__ __forceinline__ double neg(double x) { return -x; }
-__device__ __forceinline__ double quot(double a, double b) { return a / b; }
-__device__ __forceinline__ double value(double x) { return x; }
-__device__ __forceinline__ bool less(double a, double b) { return a < b; }
 __device__ __forceinline__ double shfl_xor(double x, int o) {
   return __shfl_xor_sync(0xffffffffu, x, o);
 }
@@ -166,10 +114,12 @@ template <typename TI>
 struct Wide;
 template <>
 struct Wide<float> {
-  using W = Pair;
-  static __device__ __forceinline__ Pair make(double x) {
+  using W = Tri;
+  static __device__ __forceinline__ Tri make(double x) {
     const float h = (float)x;
-    return {h, (float)(x - (double)h)};
+    x -= (double)h;
+    const float m = (float)x;
+    return {h, m, (float)(x - (double)m)};
   }
 };
 template <>
@@ -196,8 +146,9 @@ __device__ __forceinline__ double ld_peer(const double* p, uint32_t rank) {
   asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(peer(p, rank)) : "memory");
   return v;
 }
-__device__ __forceinline__ void st_peer(Pair* p, uint32_t rank, Pair v) {
-  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(peer(p, rank)), "f"(v.hi), "f"(v.lo)
+__device__ __forceinline__ void st_peer(Tri* p, uint32_t rank, Tri v) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %3};" ::"r"(peer(p, rank)), "f"(v.h),
+               "f"(v.m), "f"(v.l)
                : "memory");
 }
 __device__ __forceinline__ void st_peer(double* p, uint32_t rank, double v) {
@@ -245,7 +196,7 @@ struct Acc64 {
 // HELD: the CTA's rows of G^ are copied to shared memory; else they are streamed by
 // every product (from L2 when the batch's G^ fits it).
 template <typename TG, typename TI, bool HELD, int T>
-__global__ void __launch_bounds__(T, sizeof(TI) == 4 ? 1024 / T : 1)
+__global__ void __launch_bounds__(T, sizeof(TI) == 4 ? 768 / T : 1)
     k_inner_cluster(const InnerCta* __restrict__ ctas, const InnerGroup* __restrict__ groups,
                     const int32_t* __restrict__ cols, InnerClass C, const TG* __restrict__ ghat,
                     const double* __restrict__ g64, const double* __restrict__ z064,
@@ -417,9 +368,9 @@ __global__ void __launch_bounds__(T, sizeof(TI) == 4 ? 1024 / T : 1)
     for (int o = 16; o > 0; o >>= 1) ref2 += __shfl_xor_sync(0xffffffffu, ref2, o);
   }
   const double ref = sqrt(ref2);
-  // power of two that brings ||g|| to [1, 2) (FP32 vectors only)
+  // power of two that brings ||g|| to [2^20, 2^21) (FP32 vectors only)
   int ex = 0;
-  if (sizeof(TI) == 4 && ref > 0.0 && ref < 1e300) ex = max(-1000, min(1000, ilogb(ref)));
+  if (sizeof(TI) == 4 && ref > 0.0 && ref < 1e300) ex = max(-1000, min(1000, ilogb(ref) - 20));
   const double down = scalbn(1.0, -ex);
   W rr[1] = {};  // ||r||^2 in the vectors' precision
   for (int i = tid; i < c.nrows; i += T) {
@@ -430,7 +381,7 @@ __global__ void __launch_bounds__(T, sizeof(TI) == 4 ? 1024 / T : 1)
   }
   reduce(0, rr);
   // stop when ||r|| <= tol ||g||, as squares
-  const TI lim = (TI)(tol * tol * (down * down) * ref2);
+  const W lim = Wide<TI>::make(tol * tol * (down * down) * ref2);
   bool active = ref > 0.0 && !(outer && !outer[c.sys].active), guess = false;
   if (z064 && active) {  // the guess is taken when its residual is smaller than that of zero
     const W r0 = rr[0];
@@ -445,7 +396,7 @@ __global__ void __launch_bounds__(T, sizeof(TI) == 4 ? 1024 / T : 1)
     }
     reduce(1, rr);
     guess = less(rr[0], r0);
-    if (guess && value(rr[0]) <= lim) active = false;
+    if (guess && at_most(rr[0], lim)) active = false;
     for (int i = tid; i < c.nrows; i += T) {
       if (guess)
         r[i] = sv[i];
@@ -455,7 +406,7 @@ __global__ void __launch_bounds__(T, sizeof(TI) == 4 ? 1024 / T : 1)
     if (!guess) rr[0] = r0;
   }
   // rho = (rh, r) with rh = r; the first p is r (beta = 0)
-  W rho = rr[0], alpha = Wide<TI>::make(1.0), omega = alpha, beta{};
+  W rho = rr[0], alpha = Wide<TI>::make(1.0), omega = alpha, beta{}, bo{};  // bo = -beta omega
   bool breakdown = value(rho) == TI(0);
   double iters = 0.0;
   for (int i = tid; i < c.nrows; i += T) rh[i] = r[i];
@@ -463,9 +414,7 @@ __global__ void __launch_bounds__(T, sizeof(TI) == 4 ? 1024 / T : 1)
   for (int it = 1; active; ++it) {
     const TI *p0 = pbuf + (it & 1) * C.rows, *v0 = vbuf + (it & 1) * C.rows;
     TI *p = pbuf + (~it & 1) * C.rows, *v = vbuf + (~it & 1) * C.rows;
-    auto next_p = [&](TI rv, TI pv, TI vv) {
-      return value(add(rv, mul(beta, add(pv, neg(mul(omega, vv))))));
-    };
+    auto next_p = [&](TI rv, TI pv, TI vv) { return lin(rv, beta, pv, bo, vv); };
     for (int i = tid; i < c.nrows; i += T) p[i] = it == 1 ? r[i] : next_p(r[i], p0[i], v0[i]);
     product(p, v, [&](uint32_t rk, int i) {
       const TI rv = ld_peer(r + i, rk);
@@ -480,7 +429,8 @@ __global__ void __launch_bounds__(T, sizeof(TI) == 4 ? 1024 / T : 1)
     } else {
       alpha = quot(rho, a[0]);
     }
-    auto next_s = [&](TI rv, TI vv) { return value(add(rv, neg(mul(alpha, vv)))); };
+    const W na = neg(alpha);
+    auto next_s = [&](TI rv, TI vv) { return lin(rv, na, vv); };
     for (int i = tid; i < c.nrows; i += T) sv[i] = next_s(r[i], v[i]);
     product(sv, t, [&](uint32_t rk, int i) { return next_s(ld_peer(r + i, rk), ld_peer(v + i, rk)); });
     // (t, s), (t, t) and ||s||^2 with one barrier: the half-step check comes after
@@ -492,8 +442,8 @@ __global__ void __launch_bounds__(T, sizeof(TI) == 4 ? 1024 / T : 1)
       b[2] = sum(b[2], mul(sv[i], sv[i]));
     }
     reduce(2, b);
-    if (value(b[2]) <= lim) {  // the half step
-      for (int i = tid; i < c.nrows; i += T) z[i] = value(add(z[i], mul(alpha, p[i])));
+    if (at_most(b[2], lim)) {  // the half step
+      for (int i = tid; i < c.nrows; i += T) z[i] = lin(z[i], alpha, p[i]);
       iters = it - 0.5;
       break;
     }
@@ -502,19 +452,22 @@ __global__ void __launch_bounds__(T, sizeof(TI) == 4 ? 1024 / T : 1)
       break;
     }
     omega = value(b[1]) != TI(0) ? quot(b[0], b[1]) : W{};
+    const W ao = quot(alpha, omega);  // not used if omega is zero
     W d[2] = {};
     for (int i = tid; i < c.nrows; i += T) {
-      z[i] = value(add(z[i], add(mul(alpha, p[i]), mul(omega, sv[i]))));
-      const TI rv = value(add(sv[i], neg(mul(omega, t[i]))));
+      z[i] = lin(z[i], alpha, p[i], omega, sv[i]);
+      const TI rv = lin(sv[i], neg(omega), t[i]);
       r[i] = rv;
       d[0] = sum(d[0], mul(rv, rv));
       d[1] = sum(d[1], mul(rh[i], rv));
     }
     reduce(3, d);
     iters = it;
-    if (value(d[0]) <= lim || value(omega) == TI(0) || it >= maxit) break;
+    if (at_most(d[0], lim) || value(omega) == TI(0) || it >= maxit) break;
     breakdown = value(d[1]) == TI(0);
-    beta = mul(quot(d[1], rho), quot(alpha, omega));
+    const W ratio = quot(d[1], rho);
+    beta = mul(ratio, ao);
+    bo = neg(mul(ratio, alpha));
     rho = d[1];
   }
   const double up = scalbn(1.0, ex);
@@ -664,8 +617,8 @@ static void plan_mode(const InnerInput& in, bool held, InnerPlan& P) {
 }
 
 // Held in shared memory if every system of the handle fits a cluster (1.7 MB), however
-// many there are: G^ is read once per solve.  One system of 384 rows takes 7.8 us an
-// iteration (loop 31); 256 systems of 1,100 rows 8.0 ms per five reduced solves (loop
+// many there are: G^ is read once per solve.  One system of 384 rows takes 8.9 us an
+// iteration (loop 31); 256 systems of 1,100 rows 9.4 ms per five reduced solves (loop
 // 20.2; streamed with all systems resident 8.9, bound by reading 98 MB per product).
 // Otherwise streamed, when there are so few systems that all run at once; else
 // the plan is not ok and the loop takes them.
