@@ -270,3 +270,38 @@ def test_statistics_of_a_batch_with_an_uncoupled_system(form):
     # the uncoupled system may add outer iterations, in which the coupled one takes none
     assert both["inner_iterations"] == alone["inner_iterations"]
     assert np.array_equal(z1, z2)
+
+
+@pytest.mark.parametrize("ghat", ["FP16", "BF16", "FP32", "FP64"])
+@pytest.mark.parametrize("inner", ["FP32", "FP64"])
+def test_small_system_inner_iteration_forms_and_guess(ghat, inner):
+    """The inner iteration in one launch for every storage of G^ and precision of the vectors:
+    the residual on the stored G^ (as in test_reduced_solve_paths), and a guess of the first
+    preconditioner application -- a bad one is not used, the answer saves its iterations."""
+    if (ghat, inner) == ("FP64", "FP32"):
+        pytest.skip("an FP64 G^ needs FP64 vectors")
+    fact = dict(factor_prec=N.DDPS_FP64, spike_prec=N.DDPS_FP64) if ghat == "FP64" else \
+        dict(factor_prec=N.DDPS_FP32, spike_prec=N.DDPS_BF16X3)
+    P = W.small_convdiff_2d(40, 3, seed=2)
+    S = make_solver(P, tol_in=1e-5, maxit_in=300, tol_out=1e-10, **fact,
+                    ghat_prec=getattr(N, "DDPS_" + ghat), inner_prec=getattr(N, "DDPS_" + inner))
+    g = np.random.default_rng(9).uniform(-1, 1, S.m)
+    z = host(S.reduced_solve(dev(g)))
+    r = g - z
+    for b in range(3):
+        q0, q1, cols = S.ghat_layout(b)
+        r[q0:q1] -= S.ghat_block(b) @ z[cols]
+    assert np.linalg.norm(r) <= 1.1e-5 * np.linalg.norm(g)
+    f = dev(P.f)
+    _, cold = S.solve(f)
+    zhat, _ = S.reduced_solution()
+    S.set_reduced_guess(dev(1e3 * np.random.default_rng(3).standard_normal(S.m)))
+    x, bad = S.solve(f)
+    assert bad["guess_used"] == 0 and bad["first_inner_iters"] == cold["first_inner_iters"]
+    S.set_reduced_guess(zhat)
+    y, warm = S.solve(f)
+    assert warm["status"] == "DDPS_OK" and warm["guess_used"] == 1
+    # the guess meets the tolerance but for its own last rounding
+    assert warm["first_inner_iters"] <= 1.0 < cold["first_inner_iters"]
+    assert relerr(host(y), host(x)) <= 1e-7
+    S.close()
