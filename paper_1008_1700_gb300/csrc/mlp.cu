@@ -10,6 +10,7 @@
 #include <cstdint>
 
 #include "ddps.h"
+#include "tri.h"
 
 namespace {
 
@@ -43,27 +44,31 @@ struct GemmArgs {
   int kper;  // MODE_SPLIT: K taken by one split
 };
 
-// A sum of squares of floats as an unevaluated pair of floats (each square and
-// each sum with its rounding error, by fused multiply-add and Knuth's
-// two-sum): about 48 bits, without the FP64 pipe, whose rate is 1/64 here and
-// held the loss epilogue of a 64 x 128 tile for 4 us.
-struct Sum2 {
-  float hi = 0.f, lo = 0.f;
-  __device__ __forceinline__ void add_square(float d) {
-    const float p = d * d, e = fmaf(d, d, -p);
-    const float s = hi + p, b = s - hi;
-    lo += ((hi - (s - b)) + (p - b)) + e;
-    hi = s;
+// A sum of squares of floats as an unevaluated sum of three (tri.h): FP64's digits and more
+// without the FP64 pipe, whose rate is 1/64 here and held the loss epilogue of a 64 x 128 tile
+// for 4 us.  Squares that FP32's range does not hold to the last bit are left out and noted.
+struct SquareSum {
+  ddps::Tri t = {0.f, 0.f, 0.f};
+  bool left_out = false;
+  __device__ static __forceinline__ bool in_range(float d) {
+    return d == 0.f || (fabsf(d) >= 0x1p-48f && fabsf(d) <= 0x1p60f);
   }
+  __device__ __forceinline__ void add(float d) {
+    const bool in = in_range(d);
+    const float v = in ? d : 0.f;
+    t = ddps::sum(t, ddps::mul(v, v));
+    left_out |= !in;
+  }
+  __device__ __forceinline__ double total() const { return ((double)t.l + t.m) + t.h; }
 };
 
-__device__ __forceinline__ float finish(const GemmArgs& g, float v, int64_t o, int j, Sum2& sq) {
+__device__ __forceinline__ float finish(const GemmArgs& g, float v, int64_t o, int j, SquareSum& sq) {
   if (g.mode == MODE_BIAS) return v + g.bias[j];
   if (g.mode == MODE_BIAS_RELU) return fmaxf(v + g.bias[j], 0.f);
   if (g.mode == MODE_MASK) return g.aux[o] > 0.f ? v : 0.f;
   if (g.mode == MODE_LOSS) {
     const float d = v + g.bias[j] - g.aux[o];
-    sq.add_square(d);
+    sq.add(d);
     return d * g.scale;
   }
   return v;
@@ -75,7 +80,7 @@ __device__ __forceinline__ float finish(const GemmArgs& g, float v, int64_t o, i
 // by FP32 arithmetic.  The rows of a batch of about 100 are the short side,
 // so the tile is 64 high: two tiles waste less of it than one of 128 and a
 // remainder.  MODE_SPLIT: blockIdx.z takes K range z of kper.  At a batch of 100
-// and 256 x 32,256 weights: output layer with loss 74 us (a 64 x 64 tile kernel
+// and 256 x 32,256 weights: output layer with loss 79 us (a 64 x 64 tile kernel
 // with a separate loss pass took 197), weight gradient 57 us (99 with the bias
 // pass), input gradient 53 + 10 us in 75 splits (5,650 us in 8 CTAs without).
 constexpr int BM = 64, BN = 128, BK = 16;
@@ -176,7 +181,7 @@ __global__ void __launch_bounds__(kThreads) k_gemm_wide(GemmArgs g) {
   }
   float* __restrict__ C = g.C + (g.mode == MODE_SPLIT ? (int64_t)blockIdx.z * g.M * g.N : 0);
   const bool cvec = g.ldc % 4 == 0 && ((uintptr_t)C & 15) == 0;
-  Sum2 sum;
+  SquareSum sum;
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
     const int i = i0 + ty * 4 + u;
@@ -199,7 +204,16 @@ __global__ void __launch_bounds__(kThreads) k_gemm_wide(GemmArgs g) {
     if (ROWSUM && blockIdx.x == 0 && tx == 0) g.rowsum[i] = rs[u];
   }
   if (g.mode == MODE_LOSS) {
-    double sq = (double)sum.hi + (double)sum.lo;
+    double sq = sum.total();
+    if (sum.left_out) {  // rare
+      for (int u = 0; u < 4; ++u)
+        for (int v = 0; v < 8; ++v) {
+          const int i = i0 + ty * 4 + u, j = j0 + v / 4 * (BN / 2) + tx * 4 + v % 4;
+          if (i >= g.M || j >= g.N) continue;
+          const float d = acc[u][v] + g.bias[j] - g.aux[i * g.ldc + j];
+          if (!SquareSum::in_range(d)) sq += (double)d * d;
+        }
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
     if ((tid & 31) == 0) red[tid >> 5] = sq;
@@ -295,7 +309,7 @@ __global__ void __launch_bounds__(kThreads) k_gemm_small(GemmArgs g0, GemmArgs g
     if ((lane & 3) == 0) R[warp * SM_T + li + u] = rs[u];
   }
   __syncthreads();
-  Sum2 sq;  // no small product takes MODE_LOSS
+  SquareSum sq;  // no small product takes MODE_LOSS
   for (int e = tid; e < SM_T * SM_T; e += kThreads) {
     const int r = e / SM_T, c = e % SM_T, i = i0 + r, j = j0 + c;
     if (i >= g.M || j >= g.N) continue;

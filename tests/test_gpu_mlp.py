@@ -88,3 +88,27 @@ def test_shapes_match_oracle(d_in, hidden, layers, d_out, B):
     go = _flat(M.backward(params, X, T))
     assert np.linalg.norm(g.cpu().numpy() - go) <= 1e-5 * np.linalg.norm(go)
     assert abs(loss.item() - M.loss(params, X, T)) <= 1e-5 * M.loss(params, X, T)
+
+
+@pytest.mark.parametrize("name,size", [("ordinary", 1.0), ("tiny", 1e-21), ("huge", 3e17), ("one_square_overflows", 0.0),
+                                       ("mixed", -1.0)])
+def test_loss_keeps_fp64_sums(name, size):
+    """The loss of a network that answers 0 is the targets' mean square: the float nearest to
+    it, for any size whose mean square is a float, also where single squares are not."""
+    d_in, hidden, layers, d_out, B = 2, 16, 1, 300, 70
+    rng = np.random.default_rng(4)
+    T = rng.uniform(0.5, 1.0, (B, d_out)) * (size if size > 0 else 1.0)
+    if name == "one_square_overflows":
+        T[B // 2, d_out // 2] = 3e19
+    if name == "mixed":
+        T *= 10.0 ** rng.integers(-18, 3, T.shape)
+    T = T.astype(np.float32)
+    p = torch.zeros(N.ddps_mlp_param_count(d_in, hidden, layers, d_out), device="cuda")
+    ws = torch.empty(N.ddps_mlp_workspace_bytes(d_in, hidden, layers, d_out, B), dtype=torch.uint8,
+                     device="cuda")
+    g, loss = torch.zeros_like(p), torch.zeros(1, device="cuda")
+    N.ddps_mlp_backward(p, d_in, hidden, layers, d_out, _dev(rng.standard_normal((B, d_in))), _dev(T), B,
+                        g, loss, ws)
+    exact = 0.5 / B * np.sum(np.longdouble(T) ** 2)
+    # the rounding to a float (or to a denormal one) and FP64 sums
+    assert abs(float(loss.item()) - exact) <= (2.0 ** -24 + 1e-12) * exact + 2.0 ** -150 * 1.01
