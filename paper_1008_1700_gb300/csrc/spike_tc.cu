@@ -579,11 +579,14 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
 // problems.  Every operand is split into three bf16 parts (x = h + m + l, 24 bits, the
 // FP32 significand) and the six products of order 2^-16 and above are taken: h h, h m,
 // m h, m m, h l, l h; what is left out is below 2^-24 of a term, an FP32 rounding.
-// The tensor core adds to its accumulator with truncation, so h h has an accumulator of
-// its own (the other products, 2^-8 of it and less, share a second one) and a sum stays
-// there for 32 values of K only, then it is added to FP32 registers: the reduced solves
-// are as exact as with FP32 FMAs (residuals within 10% either way on six grids; with one
-// accumulator and 256 values those of 2-D grids were three times as large).
+// The tensor core truncates its sums, and errors of one sign add up where those of roundings
+// cancel.  So a sum stays there for 16 values of K only (h h of the second 16 goes on top of
+// the small products of all 32, 2^-8 of it and less), then it is added to FP32 registers, and
+// matrices of up to 96 columns, whose short sums take few roundings, go through FP32 FMAs
+// (fma_tile): on 2-D grids of 80, 96 and 128 lines the reduced solve has errors of 9.6e-7,
+// 8.1e-7 and 1.30e-6 from the tensor cores, 8.3e-7, 8.3e-7 and 1.66e-6 from FMAs.  On 19 grids
+// errors are 0.26 to 1.04 times those of FMAs, 0.89 in the mean; with sums of 32 values for
+// all sizes they were up to 2.2 times as large.
 // The 256 threads load and split the next 32 values of K while the MMAs of the last
 // ones run (two stages).  Bound by the splitting and the MMAs
 // (about 800 and 880 cycles per 32 values of K and tile): 4608 x 2304 x 2304 takes
@@ -606,8 +609,90 @@ __device__ __forceinline__ void split3(const float* v, unsigned char* h, unsigne
   *reinterpret_cast<uint4*>(l) = make_uint4(c[0], c[1], c[2], c[3]);
 }
 
-constexpr int GG_GROUP = 1;  // stages of 32 per tensor-memory sum
 constexpr uint32_t GG_STAGE = 6 * TC_TILE_BYTES;
+
+// One 128 x 128 tile by FP32 FMAs in the order of K: K in steps of 16 through a double buffer
+// in shared memory, 8 x 8 results per thread, as four 4 x 4 quarters, of which those outside
+// the matrix are left out.
+__device__ void fma_tile(const GemmDesc& d, int m0, int n0, float* smem) {
+  constexpr int BK = 16, LD = 128 + 4;
+  float(*As)[BK][LD] = reinterpret_cast<float(*)[BK][LD]>(smem);
+  float(*Bs)[BK][LD] = As + 2;
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  const bool lower = m0 + 64 < d.M, right = n0 + 64 < d.N;
+  // loaders: A: row tid / 2, eight values of K; B: rows tid / 32 and 8 more, four columns each
+  const int ar = tid >> 1, ak = (tid & 1) * 8, bk = tid >> 5, bc = (tid & 31) * 4;
+  float ra[8], rb[8];
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int gk = k0 + ak + q;
+      ra[q] = m0 + ar < d.M && gk < d.K ? d.A[(int64_t)(m0 + ar) * d.lda + gk] : 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int gk = k0 + bk + 8 * (q / 4), gc = n0 + bc + q % 4;
+      rb[q] = gk < d.K && gc < d.N ? d.B[(int64_t)gk * d.ldb + gc] : 0.f;
+    }
+  };
+  auto store = [&](int st) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) As[st][ak + q][ar] = ra[q];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      *reinterpret_cast<float4*>(&Bs[st][bk + 8 * h][bc]) =
+          make_float4(rb[4 * h], rb[4 * h + 1], rb[4 * h + 2], rb[4 * h + 3]);
+  };
+  float acc[2][2][4][4] = {};
+  const int nk = (d.K + BK - 1) / BK;
+  if (nk > 0) {
+    load(0);
+    store(0);
+  }
+  __syncthreads();
+  for (int kt = 0; kt < nk; ++kt) {
+    const int st = kt & 1;
+    if (kt + 1 < nk) load((kt + 1) * BK);
+#pragma unroll 4
+    for (int k = 0; k < BK; ++k)
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        if (i && !lower) continue;
+        const float4 a4 = *reinterpret_cast<const float4*>(&As[st][k][i * 64 + ty * 4]);
+        const float a[4] = {a4.x, a4.y, a4.z, a4.w};
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          if (j && !right) continue;
+          const float4 b4 = *reinterpret_cast<const float4*>(&Bs[st][k][j * 64 + tx * 4]);
+          const float b[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) acc[i][j][u][v] = fmaf(a[u], b[v], acc[i][j][u][v]);
+        }
+      }
+    if (kt + 1 < nk) store(st ^ 1);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int r = m0 + i * 64 + ty * 4 + u;
+      if (r >= d.M) continue;
+      float* __restrict__ C = d.C + (int64_t)r * d.ldc;
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          const int c = n0 + j * 64 + tx * 4 + v;
+          if (c >= d.N) continue;
+          const float x = d.alpha * acc[i][j][u][v];
+          C[c] = d.beta == 0.f ? x : fmaf(d.beta, C[c], x);
+        }
+    }
+}
+constexpr int kFmaCols = 96;  // matrices of up to so many columns take fma_tile
 
 __global__ void __launch_bounds__(TC_THREADS, 2)
     k_gemm_grouped_tc(const GemmDesc* __restrict__ D, const int32_t* __restrict__ prefix,
@@ -624,6 +709,10 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
   const int t = blockIdx.x - prefix[lo];
   const int tiles_n = (d.N + TC_BN - 1) / TC_BN;
   const int m0 = (t / tiles_n) * TC_BM, n0 = (t % tiles_n) * TC_BN;
+  if (d.tri == 0 && d.N <= kFmaCols) {
+    fma_tile(d, m0, n0, reinterpret_cast<float*>(smem));
+    return;
+  }
   if (d.tri == GEMM_TO_M || d.tri == GEMM_TO_N)
     d.K = min(d.K, (d.tri == GEMM_TO_M ? m0 : n0) + TC_BM);
   const int kfirst = d.tri == GEMM_FROM_M ? m0 : d.tri == GEMM_FROM_N ? n0 : 0;
@@ -720,36 +809,40 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
     }
     if (kt + 1 < nk) load(kt + 1);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    const bool first = kt % GG_GROUP == 0;
-    if (first && kt > 0 && !timed_out)
+    if (kt > 0 && !timed_out)
       timed_out = !mbar_wait(smem_u32(&empty[(kt - 1) & 1]), ((kt - 1) >> 1) & 1, err);
     timed_out = __syncthreads_or(timed_out);  // all threads give up together
     if (timed_out) break;
-    if (first && kt > 0) {  // the group before is complete
+    if (kt > 0) {  // the stage before is complete
       collect();
       __syncthreads();
     }
     if (tid == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t aS = sbase + st * GG_STAGE, bS = aS + 3 * TC_TILE_BYTES;
-      const uint32_t lowp = tmem + TC_BN;
+      uint64_t a[2][3], b[2][3];
 #pragma unroll
-      for (int kk = 0; kk < TC_BK / 16; ++kk) {
-        const uint32_t ko = kk * 256;
-        uint64_t a[3], b[3];
+      for (int kk = 0; kk < 2; ++kk)
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-          a[q] = make_desc(aS + q * TC_TILE_BYTES + ko, 128, kSBO);
-          b[q] = make_desc(bS + q * TC_TILE_BYTES + ko, 128, kSBO);
+          a[kk][q] = make_desc(aS + q * TC_TILE_BYTES + kk * 256, 128, kSBO);
+          b[kk][q] = make_desc(bS + q * TC_TILE_BYTES + kk * 256, 128, kSBO);
         }
-        const uint32_t more = !first || kk > 0;
-        mma_bf16(lowp, a[2], b[0], more);
-        mma_bf16(lowp, a[0], b[2], 1u);
-        mma_bf16(lowp, a[1], b[1], 1u);
-        mma_bf16(lowp, a[1], b[0], 1u);
-        mma_bf16(lowp, a[0], b[1], 1u);
-        mma_bf16(tmem, a[0], b[0], more);
+      // h h of the first 16 values; the small products, then h h of the others
+      const uint32_t rest = tmem + TC_BN;
+      mma_bf16(tmem, a[0][0], b[0][0], 0u);
+#pragma unroll
+      for (int kk = 0; kk < 2; ++kk) {
+        mma_bf16(rest, a[kk][2], b[kk][0], kk);
+        mma_bf16(rest, a[kk][0], b[kk][2], 1u);
+        mma_bf16(rest, a[kk][1], b[kk][1], 1u);
       }
+#pragma unroll
+      for (int kk = 0; kk < 2; ++kk) {
+        mma_bf16(rest, a[kk][1], b[kk][0], 1u);
+        mma_bf16(rest, a[kk][0], b[kk][1], 1u);
+      }
+      mma_bf16(rest, a[1][0], b[1][0], 1u);
       mma_commit(smem_u32(&empty[st]));
     }
   }
