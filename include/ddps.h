@@ -127,15 +127,17 @@ typedef struct {
   int32_t reduced_solver; /* ddps_reduced_solver; DIRECT needs an explicit G^ (ghat_mode 0) and
                              a chain partition, else ddps_analyze returns DDPS_ERR_INVALID_ARG */
   int32_t use_graphs;     /* 1 (default): launch sequences that repeat unchanged (the factor
-                             phase, chunks of inner iterations, a direct-mode preconditioner
-                             application) are captured into CUDA graphs on a stream of the
-                             handle at their first use and replayed afterwards; 0: plain
-                             launches.  Graphs are not used while profiling is on. */
+                             phase, the sweeps of a block solve, chunks of inner iterations, a
+                             direct-mode preconditioner application) are captured into CUDA
+                             graphs on a stream of the handle at their first use and replayed
+                             afterwards on the caller's; 0: plain launches.  Graphs are not
+                             used while profiling is on. */
   int32_t persistent_solve; /* 1 (default): the block solves (6.1, 6.5) sweep the deep levels of
-                             small fronts (at most 128 rows) in one persistent launch per sweep,
-                             fronts ordered by per-front completion flags with bounded waits
-                             (a wait that runs out makes ddps_solve return DDPS_ERR_TIMEOUT);
-                             0: one launch per tree depth */
+                             small fronts (at most 128 rows) in one persistent launch per sweep
+                             where that is the faster (as timed by the autotuner; without it,
+                             from 16,384 such fronts on), fronts ordered by per-front completion
+                             flags with bounded waits (a wait that runs out makes ddps_solve
+                             return DDPS_ERR_TIMEOUT); 0: always one launch per tree depth */
   int32_t factor_kind;    /* a ddps_factor_kind value; 0 = exact LU */
   int32_t autotune;       /* 1 (default): the first ddps_factor times every candidate launch shape
                              of each block-solve depth and sweep (warp per front, CTA per front,
