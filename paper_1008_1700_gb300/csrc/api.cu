@@ -867,7 +867,7 @@ void block_solve_impl(ddps_handle* h, const double* y, double* g, cudaStream_t s
 }
 
 // ---------------------------------------------------------------------------
-// Autotuner of the block-solve launch shapes.  For every depth and both sweeps, each candidate shape (warp per front
+// Autotuner of the block-solve launch shapes.  For the depths and both sweeps, each candidate shape (warp per front
 // when the fronts allow, one CTA with eight loads in flight, clusters of 1,
 // 2, 4 and 8 CTAs) is timed with CUDA events on the handle's own factors
 // (one untimed launch, then the mean of three), and the fastest is kept.
@@ -934,7 +934,10 @@ void autotune_block_solve(ddps_handle* h, cudaStream_t s) {
   std::lock_guard<std::mutex> lock(g_tune_mutex);
   tune_cache_read();
   bool added = false;
-  for (int L = 0; L < A.nlevels; ++L) {
+  // Depths that the persistent sweeps may take hold fronts of at most kPersistM rows: clusters
+  // of several CTAs per front are not tried there.
+  const int top = h->persist_L >= 0 ? h->persist_L : A.nlevels;
+  auto tune_depth = [&](int L) {
     const int32_t nf = A.level_ptr[L + 1] - A.level_ptr[L];
     const int32_t mm = h->split[L].max_m;
     int64_t ent = 0;
@@ -951,7 +954,7 @@ void autotune_block_solve(ddps_handle* h, cudaStream_t s) {
       if (it != g_tune_cache.end()) {
         best = it->second;
       } else {
-        for (int cfg = SOLVE_WARP; cfg <= SOLVE_CL8; ++cfg) {
+        for (int cfg = SOLVE_WARP; cfg <= (L < top ? SOLVE_CL8 : SOLVE_CL1); ++cfg) {
           if (cfg == SOLVE_WARP && mm > kPersistM) continue;
           auto run = [&]() {
             if (sweep == 0)
@@ -979,31 +982,46 @@ void autotune_block_solve(ddps_handle* h, cudaStream_t s) {
       (sweep ? h->tune_bwd : h->tune_fwd)[L] = best;
       (sweep ? h->tune_bwd_ms : h->tune_fwd_ms)[L] = best_ms;
     }
-  }
-  // both sweeps with the deep levels in persistent launches, or every level in its own
+  };
+  for (int L = 0; L < top; ++L) tune_depth(L);
+  // Both sweeps with the deep levels in persistent launches, or every level in its own.  The
+  // shapes of these are timed only where the launches of the fixed rules come near the
+  // persistent sweeps: of a batch's 70,731 fronts each takes up to a millisecond (first
+  // factorisation 220 ms with every shape at every depth, 16 so).
   if (h->persist_L >= 0) {
     const std::string key = std::string(prop.name) + "|" + std::to_string(sizeof(T)) +
                             "|persist|" + std::to_string(A.nlevels) + "|" +
                             std::to_string(h->persist_n) + "|" +
                             std::to_string(A.factor_lu_entries);
     auto it = g_tune_cache.find(key);
+    auto tune_deep = [&]() {
+      for (int L = top; L < A.nlevels; ++L) tune_depth(L);
+    };
     if (it != g_tune_cache.end()) {
       h->use_persist = it->second == 1;
+      if (!h->use_persist) tune_deep();
     } else {
-      float ms[2];
       const int64_t l0 = h->launches;
-      for (int v = 0; v < 2; ++v) {
-        h->use_persist = v == 1;
+      auto time_sweeps = [&](bool persist) {
+        h->use_persist = persist;
         sweep_launches<T>(h, w, u, s);
         CK(cudaEventRecord(e0, s));
         for (int r = 0; r < 3; ++r) sweep_launches<T>(h, w, u, s);
         CK(cudaEventRecord(e1, s));
         CK(cudaEventSynchronize(e1));
-        CK(cudaEventElapsedTime(&ms[v], e0, e1));
+        float ms = 0.f;
+        CK(cudaEventElapsedTime(&ms, e0, e1));
+        return ms;
+      };
+      const float persistent = time_sweeps(true);
+      float launches = time_sweeps(false);
+      if (launches < 1.25f * persistent) {
+        tune_deep();
+        launches = time_sweeps(false);
       }
       h->launches = l0;
       check_launch();
-      h->use_persist = ms[1] < ms[0];
+      h->use_persist = persistent < launches;
       g_tune_cache[key] = h->use_persist ? 1 : 0;
       added = true;
     }

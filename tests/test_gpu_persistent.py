@@ -74,3 +74,37 @@ def test_persistent_sweeps_match_launches_per_depth(name, prec, bound, tmp_path)
     o = DDPSOracle(p.n, p.rowptr, p.colind, p.values, p.block_ptr, spikes=False)
     y = np.random.default_rng(9).standard_normal(sum(q.n for q in probs))[:p.n]
     assert relerr(persistent["g"][0][:p.n], o.block_solve(y)) <= bound
+
+
+FIRST = r"""
+import sys, time, numpy as np, torch
+import workloads as W
+from gpu_helpers import dev
+from paper_1008_1700_gb300 import Solver, native as N
+opts = dict(factor_prec=N.DDPS_FP32, spike_prec=N.DDPS_BF16X3, ghat_prec=N.DDPS_FP16, inner_prec=N.DDPS_FP32)
+def factor_ms(probs, times):
+    S = Solver.from_systems([(q.rowptr, q.colind, q.values, q.block_ptr) for q in probs], **opts)
+    v, out = dev(S.values_host), []
+    for _ in range(times):
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        S.factor(v)
+        torch.cuda.synchronize()
+        out.append(1e3 * (time.perf_counter() - t))
+    return out
+factor_ms([W.small_convdiff_2d(12, 2)], 2)  # context, kernels
+first, _, third = factor_ms([W.small_convdiff_2d(60 + k % 60, 8) for k in range(200)], 3)
+print(first, third)
+"""
+
+
+def test_first_factorisation_of_a_batch_does_not_try_every_shape():
+    """The autotuner of a handle's first factorisation stays within a few factorisations of a
+    batch, whose depths hold tens of thousands of small fronts (every shape at every depth
+    took as long as twenty)."""
+    env = dict(os.environ, PYTHONPATH=os.pathsep.join([os.path.dirname(HERE), HERE]))
+    env.pop("DDPS_TUNE_CACHE", None)
+    r = subprocess.run([sys.executable, "-c", FIRST], check=True, env=env, timeout=300,
+                       capture_output=True, text=True)
+    first, third = (float(v) for v in r.stdout.split())
+    assert first <= 6.0 * third, (first, third)
