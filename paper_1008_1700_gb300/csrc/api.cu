@@ -55,13 +55,13 @@ size_t prec_size(int prec) { return prec == DDPS_FP64 ? 8 : (prec == DDPS_FP32 ?
 
 }  // namespace
 
-// Fronts of one depth reordered for the LU launches: `nsmall` fronts that fit
-// the shared-memory kernel, then `nlarge` others, starting at `first`.
 // FP32 fronts of more pivots get their triangular inverses by doubling on the tensor cores
 // (build_inverse_products); at up to 512 either way takes the same time within 1% of the
 // block LU (64^3, 48^3, 300k band).
 constexpr int32_t kInvTcK = 256;
 
+// Fronts of one depth reordered for the LU launches: `nsmall` fronts that fit
+// the shared-memory kernel, then `nlarge` others, starting at `first`.
 struct LevelSplit {
   int32_t first = 0, nsmall = 0, nlarge = 0, max_small_m = 0, max_m = 0;
   // multi-CTA LU of the large fronts: per panel step p (columns 32p..32p+31),
@@ -867,10 +867,10 @@ void block_solve_impl(ddps_handle* h, const double* y, double* g, cudaStream_t s
 }
 
 // ---------------------------------------------------------------------------
-// Autotuner of the block-solve launch shapes.  For the depths and both sweeps, each candidate shape (warp per front
-// when the fronts allow, one CTA with eight loads in flight, clusters of 1,
-// 2, 4 and 8 CTAs) is timed with CUDA events on the handle's own factors
-// (one untimed launch, then the mean of three), and the fastest is kept.
+// Autotuner of the block-solve launch shapes.  For every depth that gets launches of its own
+// and both sweeps, each candidate shape (warp per front when the fronts allow, one CTA with
+// eight loads in flight, clusters of 1, 2, 4 and 8 CTAs) is timed with CUDA events on the
+// handle's own factors (one untimed launch, then the mean of three), and the fastest is kept.
 // Choices are cached per process by (device, precision, sweep, front count,
 // largest front, total front entries) and, when the environment variable
 // DDPS_TUNE_CACHE names a file, read from and written to that JSON object.
@@ -1636,7 +1636,9 @@ ddps_status solve_impl(ddps_handle* h, const double* f, double* x, const double*
 // iterative reduced solve on a stored G^ of at most 32 bits (an FP64 product is bound by the
 // FP64 pipe, not by memory; systems that fit a cluster have their own launch).  Four right-hand
 // sides, 48^3 in eight slabs, FP16 G^: G^ products 14.0 -> 4.5 ms, block solves (the vectors
-// in the grid's second dimension) 4.7 -> 2.9, launches 1,484 -> 476, the solve 22.9 -> 10.0.
+// in the grid's second dimension) 4.7 -> 2.9, launches 1,484 -> 476, the solve 22.9 -> 10.0
+// (10.4 to 12.5 on other boxes, of 25.2 to 27.0).  The host-buffer entry point takes its
+// right-hand sides one after the other.
 int wide_width(ddps_handle* h, int32_t nrhs) {
   const Analysis& A = h->A;
   if (nrhs < 2 || A.c.empty() || A.ilu || h->use_direct || h->inner.ok || h->has_guess || h->wide_failed ||

@@ -34,7 +34,7 @@ namespace {
 constexpr int kMaxCs = 8;
 constexpr size_t kSmemMax = 220 * 1024;  // dynamic shared memory of a CTA
 // G^ bytes of a system that one cluster streams by every product: at 2.9 MB (200 x 200
-// grid, 10 blocks) a re-solve takes 8.4 ms, with the launch-per-step loop 11.7; at 7.9 MB
+// grid, 10 blocks) a re-solve takes 6.0 ms, with the launch-per-step loop 9.5; at 7.9 MB
 // (256 x 256, 16 blocks) 16.8 against 12.6, where the loop's products use every SM.
 constexpr int64_t kStreamMax = 4 << 20;
 
@@ -619,7 +619,8 @@ static void plan_mode(const InnerInput& in, bool held, InnerPlan& P) {
 // Held in shared memory if every system of the handle fits a cluster (1.7 MB), however
 // many there are: G^ is read once per solve.  One system of 384 rows takes 8.9 us an
 // iteration (loop 31); 256 systems of 1,100 rows 9.4 ms per five reduced solves (loop
-// 20.2; streamed with all systems resident 8.9, bound by reading 98 MB per product).
+// 20.2; streamed with all systems resident it was the slower, 8.9 ms where held took 8.0,
+// bound by reading 98 MB per product).
 // Otherwise streamed, when there are so few systems that all run at once; else
 // the plan is not ok and the loop takes them.
 void plan_inner_cluster(const InnerInput& in, InnerPlan& P) {
