@@ -1,7 +1,8 @@
-"""FP64 spike products (fixed-point digits on the tensor cores): G^ of a block whose rows
-are all interface rows, by its residual M X = R, over sizes at the edges of the 32-row and
-128-column tiles, of the 32-column stages and of the 128-value groups of K, with unknowns
-and equations in very different units (powers of two, so that they change no rounding)."""
+"""FP64 spike products: G^ of a block whose rows are all interface rows, by its residual
+M X = R, over sizes at the edges of the 32-row and 128-column tiles and of longer sums, with
+unknowns and equations in very different units (powers of two, so that they change no
+rounding), with couplings that are numerically nothing, and the relative error of its small
+entries."""
 
 import numpy as np
 import pytest
